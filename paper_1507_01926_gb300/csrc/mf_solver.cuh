@@ -1302,27 +1302,48 @@ __device__ __forceinline__ int bfs_take(const Dev &D, int v) {
   return (int)(atomicAnd(D.blab + MF_VTX(D, v), ~BQ) >> 32);
 }
 
-// Offers label l to w; true when w must join the next list.
-__device__ __forceinline__ bool bfs_offer(const Dev &D, int w, int l) {
-  const unsigned long long c = bword(l, BQ);
-  const unsigned long long old = atomicMin(D.blab + MF_VTX(D, w), c);
-  return old > c && !(old & BQ);
+// Vertices whose BFS word is final before the first offer of a single graph's
+// BFS (its seed, and its blocker if it has one; -1: none). Offers to them are
+// left out: on a grid whose every pixel has a terminal arc, half a million
+// pixels would queue their atomics at one word (a 1024x1024 image spent 0.25 ms
+// in each such level, 2.9 of its 4.5 ms).
+struct Final {
+  int a, b;
+};
+
+// Offers word c to w where `on`; the old word (0 where not offered). One
+// predicated instruction, not a branch around an atomic: the offers of one
+// thread are then in flight together and their results are waited for at the
+// first use, after the last of them was issued.
+__device__ __forceinline__ unsigned long long bfs_offer(const Dev &D, int w, unsigned long long c, bool on) {
+  unsigned long long old;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\tsetp.ne.s32 p, %3, 0;\n\tmov.u64 %0, 0;\n\t@p atom.global.min.u64 %0, [%1], %2;\n\t}"
+      : "=&l"(old)
+      : "l"(D.blab + MF_VTX(D, w)), "l"(c), "r"((int)on)
+      : "memory");
+  return old;
 }
 
-__device__ __forceinline__ void bfs_arc(const Dev &D, Shared &sh, int a, int l, bool reverse, int next) {
+// Whether an offer of c that found `old` puts the vertex on the next list.
+__device__ __forceinline__ bool bfs_won(unsigned long long old, unsigned long long c) { return old > c && !(old & BQ); }
+
+__device__ __forceinline__ void bfs_arc(const Dev &D, Shared &sh, int a, int l, bool reverse, int next, const Final &F) {
   const int w = __ldg(&D.head[MF_SLOT(D, a)]);
   const int2 x = __ldcg(&D.rr[MF_SLOT(D, a)]);
   const int cf = reverse ? x.y : x.x;
-  if (cf > 0 && bfs_offer(D, w, l)) qpush(D, sh, next, w);
+  const unsigned long long c = bword(l, BQ);
+  if (cf > 0 && w != F.a && w != F.b && bfs_won(bfs_offer(D, w, c, true), c)) qpush(D, sh, next, w);
 }
 
 // One thread, deg <= KTD, loads issued together (with `pre`, deg <= KT and the
 // heads were loaded during the last grid barrier).
 template <int KTD>
 __device__ __forceinline__ void bfs_thread(const Dev &D, Shared &sh, int beg, int deg, int l, bool reverse, int next,
-                                           bool pre) {
+                                           bool pre, const Final &F) {
   int w[KTD], cf[KTD];
-  bool got[KTD];
+  unsigned long long old[KTD];
+  const unsigned long long c = bword(l, BQ);
 #pragma unroll
   for (int i = 0; i < KTD; i++) {
     w[i] = 0;
@@ -1330,7 +1351,7 @@ __device__ __forceinline__ void bfs_thread(const Dev &D, Shared &sh, int beg, in
     if (i < deg) {
       w[i] = (pre && i < KT) ? sh.phead[i < KT ? i : 0][threadIdx.x] : __ldg(&D.head[MF_SLOT(D, beg + i)]);
       const int2 x = __ldcg(&D.rr[MF_SLOT(D, beg + i)]);
-      cf[i] = reverse ? x.y : x.x;
+      cf[i] = (reverse ? x.y : x.x) > 0 && w[i] != F.a && w[i] != F.b;
     }
   }
   if (D.bfs_hops > 1) {
@@ -1338,28 +1359,28 @@ __device__ __forceinline__ void bfs_thread(const Dev &D, Shared &sh, int beg, in
     int rb[KTD], re[KTD];
 #pragma unroll
     for (int i = 0; i < KTD; i++) {
-      got[i] = cf[i] > 0 && bfs_offer(D, w[i], l);
-      rb[i] = cf[i] > 0 ? __ldg(&D.row[MF_ROW(D, w[i])]) : 0;
-      re[i] = cf[i] > 0 ? __ldg(&D.row[MF_ROW(D, w[i] + 1)]) : 0;
+      old[i] = bfs_offer(D, w[i], c, cf[i]);
+      rb[i] = cf[i] ? __ldg(&D.row[MF_ROW(D, w[i])]) : 0;
+      re[i] = cf[i] ? __ldg(&D.row[MF_ROW(D, w[i] + 1)]) : 0;
     }
 #pragma unroll
     for (int i = 0; i < KTD; i++)
-      if (got[i]) qpush_row(D, sh, next, w[i], rb[i], re[i] - rb[i]);
+      if (bfs_won(old[i], c)) qpush_row(D, sh, next, w[i], rb[i], re[i] - rb[i]);
     return;
   }
   // all offers first (in flight together), then the appends
 #pragma unroll
-  for (int i = 0; i < KTD; i++) got[i] = cf[i] > 0 && bfs_offer(D, w[i], l);
+  for (int i = 0; i < KTD; i++) old[i] = bfs_offer(D, w[i], c, cf[i]);
 #pragma unroll
   for (int i = 0; i < KTD; i++)
-    if (got[i]) qpush(D, sh, next, w[i]);
+    if (bfs_won(old[i], c)) qpush(D, sh, next, w[i]);
 }
 
 // One BFS level: expands the list of generation gen into generation gen + 1,
 // then (D.bfs_hops > 1) up to bfs_hops - 1 more levels of the vertices this
 // CTA reached itself, while they fit one per thread.
 template <int KTD>
-__device__ void bfs_level(const Dev &D, Shared &sh, int gen, bool reverse, TStat &st) {
+__device__ void bfs_level(const Dev &D, Shared &sh, int gen, bool reverse, TStat &st, const Final &F) {
   const int next = gen + 1;
   const Sweep sw = make_sweep(sh.lq[gen % 3], sh.lqn[gen % 3], nullptr, 0, list_of(D, gen), list_count(D, sh, gen),
                               nullptr, 0);
@@ -1401,7 +1422,7 @@ __device__ void bfs_level(const Dev &D, Shared &sh, int gen, bool reverse, TStat
       __syncthreads();
       const int pv = sh.imin[0], pl = sh.imin[1];
       const int b = __ldg(&D.row[MF_ROW(D, pv)]), e = __ldg(&D.row[MF_ROW(D, pv + 1)]);
-      for (int a = b + threadIdx.x; a < e; a += blockDim.x) bfs_arc(D, sh, a, pl, reverse, next);
+      for (int a = b + threadIdx.x; a < e; a += blockDim.x) bfs_arc(D, sh, a, pl, reverse, next, F);
       __syncthreads();
     }
     for (;;) {
@@ -1412,10 +1433,10 @@ __device__ void bfs_level(const Dev &D, Shared &sh, int gen, bool reverse, TStat
       const int pl = __shfl_sync(FULL, l, leader);
       if (lane == leader) cls = 0;
       const int b = __ldg(&D.row[MF_ROW(D, pv)]), e = __ldg(&D.row[MF_ROW(D, pv + 1)]);
-      for (int a = b + lane; a < e; a += 32) bfs_arc(D, sh, a, pl, reverse, next);
+      for (int a = b + lane; a < e; a += 32) bfs_arc(D, sh, a, pl, reverse, next, F);
       __syncwarp();
     }
-    if (cls == 1) bfs_thread<KTD>(D, sh, beg, deg, l, reverse, next, pre);
+    if (cls == 1) bfs_thread<KTD>(D, sh, beg, deg, l, reverse, next, pre, F);
     __syncwarp();
   }
   // more levels inside the CTA (only on graphs whose vertices are all
@@ -1441,7 +1462,7 @@ __device__ void bfs_level(const Dev &D, Shared &sh, int gen, bool reverse, TStat
         const int l = bfs_take(D, v) + 1;
         st.scans_bfs += deg;
         st.visits_bfs++;
-        bfs_thread<KT>(D, sh, beg, deg, l, reverse, next, false);
+        bfs_thread<KT>(D, sh, beg, deg, l, reverse, next, false, F);
       }
     }
   }
@@ -1541,7 +1562,7 @@ __device__ __forceinline__ void level_done(const Dev &D, unsigned long long t0, 
 // label 1 along its arcs, one arc per thread, into generation gen + 1. Ends
 // with a grid barrier.
 static __device__ __noinline__ bool bfs_wide_level(const Dev &D, Shared &sh, int gen, int b, int e, bool reverse,
-                                                   TStat &st, int where) {
+                                                   TStat &st, int where, const Final &F) {
   const int tid = blockIdx.x * blockDim.x + threadIdx.x, nthr = gridDim.x * blockDim.x;
   const bool timer = blockIdx.x == 0 && threadIdx.x == 0;
   const unsigned long long t0 = timer ? gtimer() : 0;
@@ -1553,7 +1574,7 @@ static __device__ __noinline__ bool bfs_wide_level(const Dev &D, Shared &sh, int
     st.visits_bfs++;
   }
   for (int a = b + tid; a < e; a += nthr) {
-    bfs_arc(D, sh, a, 1, reverse, gen + 1);
+    bfs_arc(D, sh, a, 1, reverse, gen + 1, F);
     st.scans_bfs++;
   }
   phase_end(D, sh, gen + 1, 0, nullptr);
@@ -1598,6 +1619,8 @@ __device__ bool bfs(const Dev &D, Shared &sh, const int *seeds, const int *block
   // A lone seed with more arcs than a CTA has threads (the sink or the source of a single graph) is not
   // queued: its level is expanded below by the whole grid, one arc per thread, instead of by one CTA.
   int wide_b = 0, wide_e = 0;
+  Final F{-1, -1};
+  if (nterm == 1) F = Final{__ldcg(&seeds[0]), blockers ? __ldcg(&blockers[0]) : -1};
   if (nterm == 1 && !excess_seeds && !S.on) {
     const int s0 = __ldcg(&seeds[0]);
     const int b = __ldg(&D.row[MF_ROW(D, s0)]), e = __ldg(&D.row[MF_ROW(D, s0 + 1)]);
@@ -1620,7 +1643,7 @@ __device__ bool bfs(const Dev &D, Shared &sh, const int *seeds, const int *block
   const bool timer = blockIdx.x == 0 && threadIdx.x == 0;
   int depth0 = 0;
   if (wide) {
-    if (!bfs_wide_level(D, sh, gen, wide_b, wide_e, reverse, st, where)) return false;
+    if (!bfs_wide_level(D, sh, gen, wide_b, wide_e, reverse, st, where, F)) return false;
     gen++;
     depth0 = 1;
   }
@@ -1637,7 +1660,7 @@ __device__ bool bfs(const Dev &D, Shared &sh, const int *seeds, const int *block
     if (D.bfs_pull > 0 && D.bfs_hops == 1 && fcount * D.bfs_pull > D.n)
       bfs_pull_level(D, sh, gen, depth, reverse, st, S);
     else
-      bfs_level<KTD>(D, sh, gen, reverse, st);
+      bfs_level<KTD>(D, sh, gen, reverse, st, F);
     const unsigned long long t1 = timer ? gtimer() : 0;
     if (!grid_sync(D, sh, where, PF_LEVEL, gen + 1)) return false;
     gen++;
