@@ -228,7 +228,7 @@ struct Shared {
   int lk;                   // staged entries to keep in shared memory
   long long wsum;
   int imin[MAX_WARPS];
-  long long lsum[MAX_WARPS];
+  long long lsum[4 * MAX_WARPS];  // HUB_ARCS sub-chunks of a CTA-sized vertex
   int lqn[3];               // kept entries of list generation g, in lq[g % 3]
   int qbuf[QCAP];
   int qrow[MAX_BLOCK];      // BFS staging: row[v] of qbuf[i] (i < MAX_BLOCK) when known (qdeg[i] >= 0)
@@ -957,7 +957,14 @@ static __device__ void discharge_warp(const Dev &D, Shared &sh, const RoundCtx &
   __syncwarp();
 }
 
-// One CTA (all threads call), arcs in chunks of blockDim.
+// Arcs each thread of a CTA takes per chunk of a CTA-sized vertex.
+constexpr int HUB_ARCS = 4;
+
+// One CTA (all threads call), arcs in chunks of HUB_ARCS * blockDim: thread t
+// holds arcs t, t + blockDim, ... of the chunk, so that loads are coalesced and
+// the dependent loads of HUB_ARCS arcs are in flight together, and the prefix
+// sum over the chunk (arc order) needs the same CTA barriers as one arc per
+// thread would.
 static __device__ void discharge_block(const Dev &D, const RoundCtx &R, int v, int dv, int cap_v, TStat &st,
                                 long long &work, Shared &sh) {
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
@@ -973,58 +980,80 @@ static __device__ void discharge_block(const Dev &D, const RoundCtx &R, int v, i
   for (;;) {
     int newl = cap_v;
     int skipped = 0;
-    for (int c = 0; c < deg && ex > 0; c += blockDim.x) {
-      const int i = c + threadIdx.x;
-      int w = 0, rs = 0, dw = 0;
-      bool wact = false;
-      if (i < deg) {
-        w = __ldg(&D.head[MF_SLOT(D, beg + i)]);
-        rs = __ldcg(&D.rr[MF_SLOT(D, beg + i)]).x;
-        if (rs > 0) {
-          const int2 x = load_slot(D, R.p, w);
-          dw = x.x;
-          wact = x.y == R.r;
+    for (long long c = 0; c < deg && ex > 0; c += HUB_ARCS * (int)blockDim.x) {
+      int w[HUB_ARCS], rs[HUB_ARCS], dw[HUB_ARCS];
+      unsigned wact = 0, push = 0, skip = 0;  // bit u: w in the working set, arc pushable, arc skipped
+#pragma unroll
+      for (int u = 0; u < HUB_ARCS; u++) {
+        const long long i = c + u * (int)blockDim.x + (int)threadIdx.x;
+        w[u] = 0;
+        rs[u] = 0;
+        dw[u] = 0;
+        if (i < deg) {
+          w[u] = __ldg(&D.head[MF_SLOT(D, beg + i)]);
+          rs[u] = __ldcg(&D.rr[MF_SLOT(D, beg + i)]).x;
+          st.scans_dis++;
         }
       }
-      const bool resid = rs > 0;
-      const bool adm = resid && dp == dw + 1;
-      const bool skip = adm && !D.simple && wact && !wins(dv, dw, v, w);
-      const bool pushable = adm && !skip;
-      const long long pr = pushable ? (long long)rs : 0;
-      const long long incl_w = warp_incl_scan(pr, lane);
+#pragma unroll
+      for (int u = 0; u < HUB_ARCS; u++)
+        if (rs[u] > 0) {
+          const int2 x = load_slot(D, R.p, w[u]);
+          dw[u] = x.x;
+          if (x.y == R.r) wact |= 1u << u;
+          st.scans_res++;
+        }
+#pragma unroll
+      for (int u = 0; u < HUB_ARCS; u++)
+        if (rs[u] > 0 && dp == dw[u] + 1) {
+          if (!D.simple && ((wact >> u) & 1u) && !wins(dv, dw[u], v, w[u]))
+            skip |= 1u << u;
+          else
+            push |= 1u << u;
+        }
       __syncthreads();  // previous chunk finished reading sh
-      if (lane == 31) sh.lsum[wid] = incl_w;
       if (threadIdx.x == 0) sh.flag = 0;
+      long long incl[HUB_ARCS];
+#pragma unroll
+      for (int u = 0; u < HUB_ARCS; u++) {
+        const bool p = (push >> u) & 1u;
+        incl[u] = __ballot_sync(FULL, p) ? warp_incl_scan(p ? (long long)rs[u] : 0, lane) : 0;
+        if (lane == 31) sh.lsum[u * MAX_WARPS + wid] = incl[u];
+      }
       __syncthreads();
-      long long wbase = 0, total = 0;
-      for (int k = 0; k < nw; k++) {
-        long long s = sh.lsum[k];
-        if (k < wid) wbase += s;
-        total += s;
-      }
-      const long long excl = wbase + incl_w - pr;
-      long long delta = 0;
-      if (pushable && excl < ex) delta = min((long long)rs, ex - excl);
-      st.scans_dis += (i < deg ? 1 : 0);
-      st.scans_res += (resid ? 1 : 0);
-      bool found = false;
-      if (delta > 0) {
-        push_res(D, beg + i, __ldg(&D.rev[MF_SLOT(D, beg + i)]), (int)delta);
-        rs -= (int)delta;
-        st.pushes++;
-        if (dw == 0) {
-          to_sink += delta;
-          sink = w;
-        } else {
-          found = deliver(D, R, w, wact, delta);
-        }
-      }
-      if (found) qpush(D, sh, R.next, w);
-      if (resid && !skip && rs > 0 && dw >= dp) newl = min(newl, dw + 1);
       if (skip) sh.flag = 1;
+      long long base = 0;  // pushable residuals of the arcs before sub-chunk u
+#pragma unroll
+      for (int u = 0; u < HUB_ARCS; u++) {
+        long long wbase = base;
+        for (int k = 0; k < nw; k++) {
+          const long long x = sh.lsum[u * MAX_WARPS + k];
+          if (k < wid) wbase += x;
+          base += x;
+        }
+        bool found = false;
+        if ((push >> u) & 1u) {
+          const long long excl = wbase + incl[u] - rs[u];
+          const long long delta = excl < ex ? min((long long)rs[u], ex - excl) : 0;
+          if (delta > 0) {
+            const int a = (int)(beg + c) + u * (int)blockDim.x + (int)threadIdx.x;
+            push_res(D, a, __ldg(&D.rev[MF_SLOT(D, a)]), (int)delta);
+            rs[u] -= (int)delta;
+            st.pushes++;
+            if (dw[u] == 0) {
+              to_sink += delta;
+              sink = w[u];
+            } else {
+              found = deliver(D, R, w[u], (wact >> u) & 1u, delta);
+            }
+          }
+        }
+        if (found) qpush(D, sh, R.next, w[u]);
+        if (!((skip >> u) & 1u) && rs[u] > 0 && dw[u] >= dp) newl = min(newl, dw[u] + 1);
+      }
       __syncthreads();
       skipped |= sh.flag;
-      ex = total >= ex ? 0 : ex - total;
+      ex = base >= ex ? 0 : ex - base;
     }
     // block min of newl
     int wm = warp_min(newl);
@@ -1348,6 +1377,34 @@ __device__ __forceinline__ void bfs_arc(const Dev &D, Shared &sh, int a, int l, 
   if (cf > 0 && w != F.a && w != F.b && bfs_won(bfs_offer(D, w, c, true), c)) qpush(D, sh, next, w);
 }
 
+// Offers label l along the slots first, first + stride, ... below end: HUB_ARCS
+// at a time, loads and offers in flight together.
+static __device__ void bfs_arcs(const Dev &D, Shared &sh, int first, int end, int stride, int l, bool reverse, int next,
+                                const Final &F) {
+  const unsigned long long c = bword(l, BQ);
+  for (long long a = first; a < end; a += HUB_ARCS * stride) {
+    int w[HUB_ARCS];
+    bool on[HUB_ARCS];
+    unsigned long long old[HUB_ARCS];
+#pragma unroll
+    for (int u = 0; u < HUB_ARCS; u++) {
+      const long long b = a + (long long)u * stride;
+      w[u] = 0;
+      on[u] = false;
+      if (b < end) {
+        w[u] = __ldg(&D.head[MF_SLOT(D, b)]);
+        const int2 x = __ldcg(&D.rr[MF_SLOT(D, b)]);
+        on[u] = (reverse ? x.y : x.x) > 0 && w[u] != F.a && w[u] != F.b;
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < HUB_ARCS; u++) old[u] = bfs_offer(D, w[u], c, on[u]);
+#pragma unroll
+    for (int u = 0; u < HUB_ARCS; u++)
+      if (bfs_won(old[u], c)) qpush(D, sh, next, w[u]);
+  }
+}
+
 // One thread, deg <= KTD, loads issued together (with pre >= 0, deg <= KT and the
 // heads were loaded during the last grid barrier, for kept entry `pre`).
 template <int KTD>
@@ -1435,7 +1492,7 @@ __device__ void bfs_level(const Dev &D, Shared &sh, int gen, bool reverse, TStat
       __syncthreads();
       const int pv = sh.imin[0], pl = sh.imin[1];
       const int b = __ldg(&D.row[MF_ROW(D, pv)]), e = __ldg(&D.row[MF_ROW(D, pv + 1)]);
-      for (int a = b + threadIdx.x; a < e; a += blockDim.x) bfs_arc(D, sh, a, pl, reverse, next, F);
+      bfs_arcs(D, sh, b + (int)threadIdx.x, e, blockDim.x, pl, reverse, next, F);
       __syncthreads();
     }
     for (;;) {
@@ -1446,7 +1503,7 @@ __device__ void bfs_level(const Dev &D, Shared &sh, int gen, bool reverse, TStat
       const int pl = __shfl_sync(FULL, l, leader);
       if (lane == leader) cls = 0;
       const int b = __ldg(&D.row[MF_ROW(D, pv)]), e = __ldg(&D.row[MF_ROW(D, pv + 1)]);
-      for (int a = b + lane; a < e; a += 32) bfs_arc(D, sh, a, pl, reverse, next, F);
+      bfs_arcs(D, sh, b + lane, e, 32, pl, reverse, next, F);
       __syncwarp();
     }
     if (cls == 1) bfs_thread<KTD>(D, sh, beg, deg, l, reverse, next, pre ? item : -1, F);
