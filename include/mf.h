@@ -26,6 +26,16 @@
  * the call (the library copies what it needs). Output arrays are allocated by
  * the caller, except those of mf_build_csr (freed with mf_free_csr).
  *
+ * Lattices: a single graph whose vertices other than s and t, in order, are the
+ * cells of a row-major 2D or 3D box, with arcs between neighbouring cells and
+ * between cells and s or t only (at most one slot per direction and terminal,
+ * found when the graph is created), is solved by mf_solve / mf_solve_device on
+ * tiles of cells instead of vertex lists, where its options ask for nothing
+ * that only the list solver has: simple_rounds, gap_every and max_rounds 0,
+ * gr_time_ratio > 0, block_threads 256, kernel_variant 0, local_lists on. Of the
+ * options it then takes gr_time_ratio (its only relabel trigger), cut_only,
+ * use_graph, timeout_ms and blocks_per_sm (2D). Same value and cut.
+ *
  * Errors: every int-returning call returns MF_OK (0), MF_PENDING (1, only
  * mf_poll) or a negative MF_ERR_* code; mf_last_error() then describes the
  * last failure of the calling thread. Calls on one mf_graph must not overlap;
@@ -166,7 +176,9 @@ typedef struct mf_options {
 /* Counters of the last solve. Arc scans count every slot examined by a
  * discharge pass (a relabel pass of the simple rounds) or a BFS expansion,
  * slots with zero residual included; scans_discharge_residual counts the
- * discharge scans of slots with positive residual. */
+ * discharge scans of slots with positive residual. Of a lattice solve, rounds and
+ * bfs_levels count sweeps over the tiles (2D) or visits of tiles (3D), the other
+ * counters cells and their slots; the CTA 0 times and rounds_by_size stay 0. */
 typedef struct mf_stats {
   int64_t rounds;           /* push-relabel rounds, both phases */
   int64_t rounds_phase1;
@@ -274,7 +286,7 @@ int mf_solve(mf_graph *g, int64_t *flow_value, int32_t *arc_flow, uint32_t *cut_
  * returns after the solve finished (it reads the status word back). */
 int mf_solve_device(mf_graph *g, void *stream, int64_t *d_flow_value, int32_t *d_arc_flow, uint32_t *d_cut_bits);
 
-/* Tracing: solves g like mf_solve (no outputs) and records, for each of the
+/* Tracing: solves g by the list solver (no outputs) and records, for each of the
  * first `capacity` push-relabel rounds of both phases, the working-set size
  * (live[k]) and whether a global relabel ran right before the round
  * (relabel_before[k] = 1), and for each of the first `level_capacity` BFS

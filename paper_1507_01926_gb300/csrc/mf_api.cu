@@ -153,7 +153,7 @@ static void free_graph_buffers(mf_graph *g) {
   void *ps[] = {g->row, g->head, g->rev, g->cap, g->rr, g->vs, g->blab, g->list[0], g->list[1], g->list[2],
                 g->src, g->snk, g->ctl, g->d_value, g->d_flow, g->d_cut, g->vinst, g->hist,
                 g->tiles, g->voff, g->live, g->cwoff, g->d_cutw, g->inst, g->inst_work, g->inst_marcs, g->carry,
-                g->gseed, g->gblocker};
+                g->gseed, g->gblocker, g->lat_buf};
   for (void *p : ps) gfree(g, p);
   if (g->gexec) cudaGraphExecDestroy(g->gexec);
   if (!g->lane_host) {
@@ -244,10 +244,12 @@ int validate_on_device(mf_graph *g, const long long *row64, const long long *rev
       return cuda_fail(e, "graph validation");
     }
   }
-  gfree(g, flags);
   g->m_arcs = (long long)((unsigned long long)h[2] | ((unsigned long long)h[3] << 32));
   g->max_degree = h[1];
-  return flags_to_status(h[0]);
+  int rc = flags_to_status(h[0]);
+  if (rc == MF_OK) rc = lattice_detect(g, reinterpret_cast<int *>(flags), st);
+  gfree(g, flags);
+  return rc;
 }
 
 int launch_config(mf_graph *g) {
@@ -261,7 +263,7 @@ int launch_config(mf_graph *g) {
   if (g->opt.blocks_per_sm > 0 && g->opt.blocks_per_sm < bps) bps = g->opt.blocks_per_sm;
   g->grid = bps * prop.multiProcessorCount;
   g->block = g->opt.block_threads;
-  return MF_OK;
+  return g->lat.dim ? lattice_grid(g, prop.multiProcessorCount, &g->lat_grid) : MF_OK;
 }
 
 int check_options(const mf_options *o) {
@@ -362,7 +364,9 @@ static cudaError_t enqueue_solve(mf_graph *g, const Dev &D, cudaStream_t st, boo
   cudaError_t e;
   if ((e = cudaMemsetAsync(g->ctl, 0, sizeof(Ctl), st)) != cudaSuccess) return e;
   if (timed && (e = cudaEventRecord(g->ev0, st)) != cudaSuccess) return e;
-  if ((e = launch_solver(D, g->grid, g->block, st, g->opt.kernel_variant)) != cudaSuccess) return e;
+  e = D.lat.dim ? launch_lattice(D, g->lat_grid, st) : launch_solver(D, g->grid, g->block, st, g->opt.kernel_variant);
+  if (e != cudaSuccess) return e;
+  g->ran_grid = D.lat.dim ? g->lat_grid : g->grid;
   if (timed && (e = cudaEventRecord(g->ev1, st)) != cudaSuccess) return e;
   return cudaMemcpyAsync(g->h_ctl, g->ctl, sizeof(Ctl), cudaMemcpyDeviceToHost, st);
 }
@@ -458,7 +462,7 @@ int finish_kernel(mf_graph *g) {
   s.level_work_ms = (double)c.t_lwork * 1e-6;
   s.level_wait_ms = (double)c.t_lwait * 1e-6;
   s.preflow_ms = c.t_preflow > c.t_start ? (double)(c.t_preflow - c.t_start) * 1e-6 : 0.0;
-  s.grid_blocks = g->grid;
+  s.grid_blocks = g->ran_grid;
   s.block_threads = g->block;
   s.gap_lifted = c.gap_lifted;
   s.scans_discharge_residual = c.scans_res;
@@ -637,6 +641,7 @@ void mf_destroy_graph(mf_graph *g) {
 static int solve_into(mf_graph *g, cudaStream_t st, int64_t *d_value, int32_t *d_flow, uint32_t *d_cut) {
   if (g->opt.cut_only && d_flow) return fail(MF_ERR_INVALID_ARG, "cut_only solves produce no per-arc flow");
   Dev D = make_dev(g);
+  if (lattice_applies(g)) D.lat = g->lat;
   D.out_value = d_value ? reinterpret_cast<long long *>(d_value) : g->d_value;
   D.out_flow = d_flow;
   D.out_cut = d_cut;

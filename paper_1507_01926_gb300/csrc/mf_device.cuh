@@ -49,6 +49,7 @@ struct Ctl {
   int ph2_started;        // unions: a relabel ended the preflow of some instances (they need a relabel from s)
   int cut_pending;        // unions: a relabel ended the flow phase of some instances (they need their cut)
   int done_cnt;           // unions: instances whose results are written
+  int qhead[4], qtail[4], qidle[4];  // lattice solves: tickets taken, entries made and warps waiting, by phase % 4
   long long bad_index;    // builds with MF_CHECK_BOUNDS: the first gather index found outside its array
 };
 // the kernel reads cnt as one int4 and gr_req as one int2
@@ -83,6 +84,27 @@ struct __align__(32) VRec {
   long long exc, added;
 };
 static_assert(sizeof(VRec) == 32, "one sector per vertex");
+
+// A lattice graph (mf_lattice.cu): the vertices other than s and t, in order,
+// are the cells of a row-major box X x Y x Z (Z = 1 in 2D, the last row or plane
+// may be cut short), cut into TX x TY x TZ tiles of 512 cells. Per-cell arrays
+// hold a tile's cells together.
+struct Lat {
+  int dim;             // 2, 3; 0: not a lattice
+  int X, Y, Z;
+  int TX, TY, TZ, tiles;
+  int s, t, cells;
+  long long *ex;       // excess
+  int *d;              // labels
+  int *drain, *back;   // residuals toward t and toward s
+  int *r;              // residuals per tile, direction and cell
+  int *inbox;          // per tile, face and face entry: amounts pushed over that face, not taken in yet
+  unsigned char *mask; // per cell, bit j: residual in direction j (set by a global relabel)
+  unsigned char *ret;  // per cell: excess was returned to s; then the mask of the cut
+  int *list[2];        // 2D: tile lists by generation parity; 3D: tile queues by phase parity
+  int *state;          // per tile. 2D: last sweep it was queued for; 3D: queued, running, faces with an inbox
+  int *bits;           // 2D: 2 x tiles, by sweep parity: faces whose inbox holds something
+};
 
 // Device view of one (possibly multi-instance) graph.
 //
@@ -164,6 +186,7 @@ struct Dev {
   int *trace_lv;          // nullable: frontier size of every BFS level, in order
   int *trace_lv_ns;       // nullable: ns of every BFS level (CTA 0, to the end of its grid barrier)
   long long trace_lv_cap;
+  Lat lat;                // lattice solves (dim 0: the list solver runs)
   // outputs (device pointers, each nullable)
   long long *out_value;   // per instance
   int *out_flow;          // m

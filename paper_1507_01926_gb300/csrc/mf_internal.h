@@ -18,6 +18,10 @@ struct mf_graph {
   mf_options opt{};
   mf_stats stats{};
   int grid = 0, block = 0;
+  mf::Lat lat{};               // lattice graphs: geometry and state (dim 0: not a lattice)
+  void *lat_buf = nullptr;     // the lattice state, where it does not fit the list solver's arrays
+  int lat_grid = 0;            // CTAs of a lattice solve
+  int ran_grid = 0;            // CTAs of the last solve
   // device state
   int *row = nullptr, *head = nullptr, *rev = nullptr, *cap = nullptr;
   int2 *rr = nullptr;
@@ -91,6 +95,10 @@ int solver_variant_max_threads(int variant);
 int solver_variant_max_bin_thread(int variant);
 int solver_occupancy(int block_threads, int *blocks_per_sm, int variant, bool multi);
 cudaError_t launch_solver(const Dev &D, int grid, int block, cudaStream_t stream, int variant);
+int lattice_detect(mf_graph *g, int *scratch, cudaStream_t st);
+int lattice_grid(const mf_graph *g, int sms, int *grid);
+bool lattice_applies(const mf_graph *g);
+cudaError_t launch_lattice(const Dev &D, int grid, cudaStream_t stream);
 int set_options(mf_graph *g, const mf_options *o);
 int autotune(mf_graph *g, const mf_tune_spec *spec, mf_options *best, double *best_ms);
 }  // namespace mf

@@ -25,6 +25,7 @@ namespace {
 // *ms = device time of the kernel.
 int timed_solve(mf_graph *g, double *ms, std::vector<long long> *values) {
   Dev D = make_dev(g);
+  if (lattice_applies(g)) D.lat = g->lat;
   D.out_value = g->d_value;
   int rc = run_kernel(g, D, g->stream);
   if (rc) return rc;
