@@ -7,7 +7,7 @@
 namespace mf {
 
 // Vertices per tile of a multi-instance graph (Dev::tiles).
-constexpr int TILE_VERTICES = 4096;
+constexpr int TILE_VERTICES = 1024;
 
 // Sentinel label of a vertex not yet reached by a BFS; a source-role vertex
 // carries UNV + 1 during a BFS so that it is never discovered.
@@ -50,6 +50,7 @@ struct Ctl {
   int cut_pending;        // unions: a relabel ended the flow phase of some instances (they need their cut)
   int done_cnt;           // unions: instances whose results are written
   int qhead[4], qtail[4], qidle[4];  // lattice solves: tickets taken, entries made and warps waiting, by phase % 4
+  int runs;               // unions: runs of arcs of the seeds a BFS does not queue
   long long bad_index;    // builds with MF_CHECK_BOUNDS: the first gather index found outside its array
 };
 // the kernel reads cnt as one int4 and gr_req as one int2

@@ -1343,14 +1343,28 @@ __device__ __forceinline__ int bfs_take(const Dev &D, int v) {
   return (int)(atomicAnd(D.blab + MF_VTX(D, v), ~BQ) >> 32);
 }
 
-// Vertices whose BFS word is final before the first offer of a single graph's
-// BFS (its seed, and its blocker if it has one; -1: none). Offers to them are
-// left out: on a grid whose every pixel has a terminal arc, half a million
-// pixels would queue their atomics at one word (a 1024x1024 image spent 0.25 ms
-// in each such level, 2.9 of its 4.5 ms).
+// Vertices whose BFS word is final before the first offer: the seed of the BFS
+// (of the vertex's instance, in a union), and its blocker if it has one (-1:
+// none). Offers to them are left out: on a grid whose every pixel has a terminal
+// arc, half a million pixels would queue their atomics at one word (a 1024x1024
+// image spent 0.25 ms in each such level, 2.9 of its 4.5 ms).
 struct Final {
   int a, b;
 };
+
+// What a BFS runs from and around, one entry per instance (read through L2: a
+// union's change during the launch).
+struct Ends {
+  const int *seeds, *blockers;  // blockers nullable
+};
+
+// Final of vertex v. `one`: that of a single graph's BFS.
+template <bool MULTI>
+__device__ __forceinline__ Final final_of(const Dev &D, const Ends &E, const Final &one, int v) {
+  if (!MULTI) return one;
+  const int k = __ldg(&D.vinst[v]).y;
+  return Final{__ldcg(&E.seeds[k]), E.blockers ? __ldcg(&E.blockers[k]) : -1};
+}
 
 // Offers word c to w where `on`; the old word (0 where not offered). One
 // predicated instruction, not a branch around an atomic: the offers of one
@@ -1448,9 +1462,16 @@ __device__ __forceinline__ void bfs_thread(const Dev &D, Shared &sh, int beg, in
 // One BFS level: expands the list of generation gen into generation gen + 1,
 // then (D.bfs_hops > 1) up to bfs_hops - 1 more levels of the vertices this
 // CTA reached itself, while they fit one per thread.
-template <int KTD>
-__device__ void bfs_level(const Dev &D, Shared &sh, int gen, bool reverse, TStat &st, const Final &F) {
+template <int KTD, bool MULTI>
+__device__ void bfs_level(const Dev &D, Shared &sh, int gen, bool reverse, TStat &st, const Ends &E, const Final &one,
+                          int runs) {
   const int next = gen + 1;
+  if (MULTI)  // level 0 of the union's seeds with many arcs
+    for (int i = blockIdx.x; i < runs; i += gridDim.x) {
+      const int a = __ldcg(&list_of(D, gen + 2)[2 * i]), e = __ldcg(&list_of(D, gen + 2)[2 * i + 1]);
+      bfs_arcs(D, sh, a + (int)threadIdx.x, e, blockDim.x, 1, reverse, next, Final{-1, -1});
+      if (threadIdx.x == 0) st.scans_bfs += e - a;
+    }
   const Sweep sw = make_sweep(sh.lq[gen % 3], sh.lqn[gen % 3], nullptr, 0, list_of(D, gen), list_count(D, sh, gen),
                               nullptr, 0);
   if (blockIdx.x == 0 && threadIdx.x == 0) {
@@ -1463,9 +1484,11 @@ __device__ void bfs_level(const Dev &D, Shared &sh, int gen, bool reverse, TStat
     const int item = sweep_pos(off, sw.items);
     if (sweep_item(sw, item, v) != 1) v = -1;
     int beg = 0, deg = 0, cls = 0, l = 0;
+    Final F{-1, -1};
     const bool pre = v >= 0 && item < (int)blockDim.x && sh.pv[item] == v;  // row and heads loaded during the last grid barrier
     if (v >= 0) {
       l = bfs_take(D, v) + 1;
+      F = final_of<MULTI>(D, E, one, v);
       if (pre) {
         beg = sh.pbeg[item];
         deg = sh.pdeg[item];
@@ -1488,11 +1511,14 @@ __device__ void bfs_level(const Dev &D, Shared &sh, int gen, bool reverse, TStat
         cls = 0;
         sh.imin[0] = v;
         sh.imin[1] = l;
+        sh.imin[2] = F.a;
+        sh.imin[3] = F.b;
       }
       __syncthreads();
       const int pv = sh.imin[0], pl = sh.imin[1];
+      const Final pF{sh.imin[2], sh.imin[3]};
       const int b = __ldg(&D.row[MF_ROW(D, pv)]), e = __ldg(&D.row[MF_ROW(D, pv + 1)]);
-      bfs_arcs(D, sh, b + (int)threadIdx.x, e, blockDim.x, pl, reverse, next, F);
+      bfs_arcs(D, sh, b + (int)threadIdx.x, e, blockDim.x, pl, reverse, next, pF);
       __syncthreads();
     }
     for (;;) {
@@ -1501,9 +1527,10 @@ __device__ void bfs_level(const Dev &D, Shared &sh, int gen, bool reverse, TStat
       const int leader = __ffs(mm) - 1;
       const int pv = __shfl_sync(FULL, v, leader);
       const int pl = __shfl_sync(FULL, l, leader);
+      const Final pF{__shfl_sync(FULL, F.a, leader), __shfl_sync(FULL, F.b, leader)};
       if (lane == leader) cls = 0;
       const int b = __ldg(&D.row[MF_ROW(D, pv)]), e = __ldg(&D.row[MF_ROW(D, pv + 1)]);
-      bfs_arcs(D, sh, b + lane, e, 32, pl, reverse, next, F);
+      bfs_arcs(D, sh, b + lane, e, 32, pl, reverse, next, pF);
       __syncwarp();
     }
     if (cls == 1) bfs_thread<KTD>(D, sh, beg, deg, l, reverse, next, pre ? item : -1, F);
@@ -1533,7 +1560,7 @@ __device__ void bfs_level(const Dev &D, Shared &sh, int gen, bool reverse, TStat
         const int l = bfs_take(D, v) + 1;
         st.scans_bfs += deg;
         st.visits_bfs++;
-        bfs_thread<KT>(D, sh, beg, deg, l, reverse, next, -1, F);
+        bfs_thread<KT>(D, sh, beg, deg, l, reverse, next, -1, final_of<MULTI>(D, E, one, v));
       }
     }
   }
@@ -1628,6 +1655,18 @@ __device__ __forceinline__ void level_done(const Dev &D, unsigned long long t0, 
   D.ctl->t_lwait += t2 - t1;
 }
 
+// Seeds of a union with more arcs than a CTA has threads (the terminals of its
+// images: one CTA walked the 115,000 arcs of a 14-frame video's sink in 0.45 ms,
+// in every relabel) are not queued: their arcs are cut into runs that the CTAs
+// share in the first level. The runs {first, end} are kept in the list of
+// generation gen + 2, which is not in use then; unions whose lists could not hold
+// them (few vertices with very many arcs) queue all seeds.
+constexpr int RUN_ARCS = 1024;
+
+__device__ __forceinline__ bool runs_fit(const Dev &D) {
+  return 2LL * ((long long)D.m / RUN_ARCS + 2LL * D.ninst) <= D.n;
+}
+
 // Level 0 of a BFS from one seed with many arcs (slots [b, e)), the seed
 // labelled 0 and not queued (generation gen is empty): the whole grid offers
 // label 1 along its arcs, one arc per thread, into generation gen + 1. Ends
@@ -1661,7 +1700,7 @@ static __device__ __noinline__ bool bfs_wide_level(const Dev &D, Shared &sh, int
 // return the last list generation (gen) is empty and no vertex is queued.
 // With S.on only the live instances take part (seeds, blockers and labels of
 // the others are left as they are; no arc leads into them).
-template <int KTD>
+template <int KTD, bool MULTI>
 __device__ bool bfs(const Dev &D, Shared &sh, const int *seeds, const int *blockers, int nterm, bool reverse,
                     bool excess_seeds, int &gen, TStat &st, int where, const Sel &S = Sel{false, 0}) {
   const int tid = blockIdx.x * blockDim.x + threadIdx.x, nthr = gridDim.x * blockDim.x;
@@ -1670,7 +1709,9 @@ __device__ bool bfs(const Dev &D, Shared &sh, const int *seeds, const int *block
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     D.ctl->cnt[(gen + 2) & 3] = 0;
     D.ctl->lcnt[(gen + 2) & 3] = 0;
+    D.ctl->runs = 0;
   }
+  const bool in_runs = MULTI && runs_fit(D);
   for_covered(D, S, [&](int v, bool valid) {
     if (!valid) return;
     unsigned long long x = bword(UNV, 0);
@@ -1687,12 +1728,12 @@ __device__ bool bfs(const Dev &D, Shared &sh, const int *seeds, const int *block
   if (!grid_sync(D, sh, where)) return false;
   // phase B: terminals (seeds join generation gen + 1 as well)
   // (seeds and blockers are read through L2: a union's per-instance seeds change during the launch)
-  // A lone seed with more arcs than a CTA has threads (the sink or the source of a single graph) is not
-  // queued: its level is expanded below by the whole grid, one arc per thread, instead of by one CTA.
+  // A single graph's seed with more arcs than a CTA has threads is not queued: its level is expanded below
+  // by the whole grid, one arc per thread, instead of by one CTA (a union's: see RUN_ARCS).
   int wide_b = 0, wide_e = 0;
   Final F{-1, -1};
-  if (nterm == 1) F = Final{__ldcg(&seeds[0]), blockers ? __ldcg(&blockers[0]) : -1};
-  if (nterm == 1 && !excess_seeds && !S.on) {
+  if (!MULTI) F = Final{__ldcg(&seeds[0]), blockers ? __ldcg(&blockers[0]) : -1};
+  if (!MULTI && !excess_seeds && !S.on) {
     const int s0 = __ldcg(&seeds[0]);
     const int b = __ldg(&D.row[MF_ROW(D, s0)]), e = __ldg(&D.row[MF_ROW(D, s0 + 1)]);
     if (e - b > (int)blockDim.x) {
@@ -1703,14 +1744,27 @@ __device__ bool bfs(const Dev &D, Shared &sh, const int *seeds, const int *block
   const bool wide = wide_e > wide_b;  // the same in every thread
   for (int i = tid; i < nterm; i += nthr) {
     if (S.on && __ldcg(&D.live[i]) != S.epoch) continue;
-    D.blab[MF_VTX(D, __ldcg(&seeds[i]))] = bword(0, wide ? 0 : BQ);
+    const int v = __ldcg(&seeds[i]);
+    bool queued = !wide;
+    if (MULTI && in_runs) {
+      const int b = __ldg(&D.row[MF_ROW(D, v)]), e = __ldg(&D.row[MF_ROW(D, v + 1)]);
+      if (e - b > (int)blockDim.x) {
+        queued = false;
+        int at = atomicAdd(&D.ctl->runs, (e - b + RUN_ARCS - 1) / RUN_ARCS);
+        for (int a = b; a < e; a += RUN_ARCS, at++) {
+          list_of(D, gen + 3)[2 * at] = a;  // gen + 2 of the level loop's first generation
+          list_of(D, gen + 3)[2 * at + 1] = min(e - a, RUN_ARCS) + a;
+        }
+        st.visits_bfs++;
+      }
+    }
+    D.blab[MF_VTX(D, v)] = bword(0, queued ? BQ : 0);
     if (blockers) D.blab[MF_VTX(D, __ldcg(&blockers[i]))] = bword(0, BB);
+    if (queued) append(D, next, v);
   }
-  if (blockIdx.x == 0 && !wide)
-    for (int i = threadIdx.x; i < nterm; i += blockDim.x)
-      if (!S.on || __ldcg(&D.live[i]) == S.epoch) append(D, next, __ldcg(&seeds[i]));
   if (!grid_sync(D, sh, where)) return false;
   gen++;
+  int runs = in_runs ? __ldcg(&D.ctl->runs) : 0;  // (written before the barrier, reset after several more)
   const bool timer = blockIdx.x == 0 && threadIdx.x == 0;
   int depth0 = 0;
   if (wide) {
@@ -1720,7 +1774,7 @@ __device__ bool bfs(const Dev &D, Shared &sh, const int *seeds, const int *block
   }
   for (int depth = depth0;; depth++) {
     const long long fcount = gen_total(D, sh, gen);
-    if (fcount == 0) break;
+    if (fcount == 0 && runs == 0) break;
     if (timer && D.trace_lv) {
       const long long k = D.ctl->levels;
       if (k < D.trace_lv_cap) D.trace_lv[k] = (int)fcount;
@@ -1728,10 +1782,11 @@ __device__ bool bfs(const Dev &D, Shared &sh, const int *seeds, const int *block
     const unsigned long long t0 = timer ? gtimer() : 0;
     // bottom-up when the frontier holds more than n / bfs_pull vertices (only for level-synchronous
     // BFS, where every frontier vertex carries the label `depth`)
-    if (D.bfs_pull > 0 && D.bfs_hops == 1 && fcount * D.bfs_pull > D.n)
+    if (D.bfs_pull > 0 && D.bfs_hops == 1 && fcount * D.bfs_pull > D.n && runs == 0)
       bfs_pull_level(D, sh, gen, depth, reverse, st, S);
     else
-      bfs_level<KTD>(D, sh, gen, reverse, st, F);
+      bfs_level<KTD, MULTI>(D, sh, gen, reverse, st, Ends{seeds, blockers}, F, runs);
+    runs = 0;
     const unsigned long long t1 = timer ? gtimer() : 0;
     if (!grid_sync(D, sh, where, PF_LEVEL, gen + 1)) return false;
     gen++;
@@ -1768,7 +1823,7 @@ __device__ bool global_relabel(const Dev &D, Shared &sh, const int *sinks, const
         I->act = 0;
       }
   }
-  if (!bfs<KTD>(D, sh, sinks, sources, D.ninst, true, false, gen, st, 2, S)) return false;
+  if (!bfs<KTD, MULTI>(D, sh, sinks, sources, D.ninst, true, false, gen, st, 2, S)) return false;
   const int next = gen + 1;
   const int p = r & 1;
   if (blockIdx.x == 0 && threadIdx.x == 0) {
@@ -2053,7 +2108,7 @@ __device__ __noinline__ bool union_cut(const Dev &D, Shared &sh, int &gen, TStat
     for (int i = threadIdx.x; i < sh.lqn[gen % 3]; i += blockDim.x) carry_push(D, lq[i]);
   }
   if (!grid_sync(D, sh, 9)) return false;
-  if (!bfs<KTD>(D, sh, D.src, nullptr, D.ninst, false, false, gen, st, 9, S)) return false;
+  if (!bfs<KTD, true>(D, sh, D.src, nullptr, D.ninst, false, false, gen, st, 9, S)) return false;
   long long left = 0;
   for (int t = blockIdx.x; t < D.ntiles; t += gridDim.x) {
     const int4 T = __ldg(&D.tiles[t]);
@@ -2287,7 +2342,7 @@ __device__ __forceinline__ void solve_body(const Dev &D) {
     }
     if (D.cut_only) {
       // S_min from the maximum preflow: reachable from s and every excess vertex.
-      ok = bfs<KTD>(D, sh, D.src, nullptr, D.ninst, false, true, gen, st, 6);
+      ok = bfs<KTD, MULTI>(D, sh, D.src, nullptr, D.ninst, false, true, gen, st, 6);
     } else {
       // Phase 2: return the excess that cannot reach t to s (s plays the sink).
       ok = run_phase<KTD, MULTI>(D, sh, D.src, D.snk, r, gen, rnd, false, st, epoch);
@@ -2306,7 +2361,7 @@ __device__ __forceinline__ void solve_body(const Dev &D) {
         }
       }
       // Cut: BFS from s over arcs with positive residual.
-      if (ok) ok = bfs<KTD>(D, sh, D.src, nullptr, D.ninst, false, false, gen, st, 9);
+      if (ok) ok = bfs<KTD, MULTI>(D, sh, D.src, nullptr, D.ninst, false, false, gen, st, 9);
     }
     if (ok) {
       if (D.out_cut) {
