@@ -135,7 +135,7 @@ typedef struct mf_options {
    * block_threads. While thread 0 of a CTA waits at the grid barrier before
    * such a round or level, its other threads load the row offsets and arc
    * heads of their kept vertices and pull the rest of their data into L2.
-   * No effect with simple_rounds. Results are the same for every setting. */
+   * Results are the same for every setting. */
   int32_t local_lists;
   /* Global relabels and cut BFS: with local_lists active, a CTA expands the
    * vertices it reached itself for up to bfs_hops levels per grid barrier

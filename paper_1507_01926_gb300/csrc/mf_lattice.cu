@@ -123,7 +123,7 @@ static int lattice_place(mf_graph *g, Lat &L) {
 // another CTA size, register budget or degree bin) runs there.
 bool lattice_applies(const mf_graph *g) {
   const mf_options &o = g->opt;
-  return g->lat.dim && !o.gap_every && o.max_rounds == 0 && o.gr_time_ratio > 0 && o.block_threads == LT &&
+  return g->lat.dim && !o.simple_rounds && !o.gap_every && o.max_rounds == 0 && o.gr_time_ratio > 0 && o.block_threads == LT &&
          o.kernel_variant == 0 && keep_local_limit(o, g->max_degree, o.block_threads) > 0;
 }
 

@@ -45,7 +45,7 @@ int solver_variant_max_bin_thread(int variant) {
 }
 
 int keep_local_limit(const mf_options &o, long long max_degree, int block_threads) {
-  if (!o.local_lists || o.simple_rounds) return 0;
+  if (!o.local_lists) return 0;
   if (max_degree > o.bin_thread || max_degree > KT) return 0;  // not every vertex is thread-sized
   const int k = o.local_lists == 1 ? block_threads / 2 : o.local_lists;
   return k < block_threads ? k : block_threads;  // block_threads <= MAX_BLOCK

@@ -226,6 +226,7 @@ struct Shared {
   int qbase;
   int qk;                   // staged entries to publish to the list in global memory
   int lk;                   // staged entries to keep in shared memory
+  int lq0;                  // entries of the generation kept before
   long long wsum;
   int imin[MAX_WARPS];
   long long lsum[4 * MAX_WARPS];  // HUB_ARCS sub-chunks of a CTA-sized vertex
@@ -297,18 +298,21 @@ __device__ __forceinline__ int sweep_pos(int off, int items) {
 // (nullable). At most D.keep_local staged entries stay in the CTA's shared
 // memory (lq[gen % 3]; their number is added to lcnt), more are published to
 // the list in global memory with one atomic for the space. Every generation is
-// staged by exactly one phase. Two CTA barriers; the next phase starts after a
-// grid barrier, which begins with a CTA barrier.
-static __device__ void phase_end(const Dev &D, Shared &sh, int gen, long long work, long long *work_dst) {
+// staged by exactly one phase, or by two (`second`: the kept entries of the
+// first stay, the second's join them where all fit). Two CTA barriers; the next
+// phase starts after a grid barrier, which begins with a CTA barrier.
+static __device__ void phase_end(const Dev &D, Shared &sh, int gen, long long work, long long *work_dst,
+                                 bool second = false) {
   const long long w = warp_sum(work);
   if ((threadIdx.x & 31) == 0 && w) atomicAdd(reinterpret_cast<unsigned long long *>(&sh.wsum), (unsigned long long)w);
   __syncthreads();
   if (threadIdx.x == 0) {
-    const int k = min(sh.qn, QCAP);
-    const bool keep = sh.qn <= D.keep_local;  // keep_local <= MAX_BLOCK < QCAP: nothing overflowed
+    const int k = min(sh.qn, QCAP), k0 = second ? sh.lqn[gen % 3] : 0;
+    const bool keep = k0 + sh.qn <= D.keep_local;  // keep_local <= MAX_BLOCK < QCAP: nothing overflowed
     sh.qk = keep ? 0 : k;
     sh.lk = keep ? k : 0;
-    sh.lqn[gen % 3] = keep ? k : 0;
+    sh.lq0 = k0;
+    sh.lqn[gen % 3] = k0 + (keep ? k : 0);
     if (!keep && k > 0) sh.qbase = atomicAdd(&D.ctl->cnt[gen & 3], k);
     if (keep && k > 0) atomicAdd(&D.ctl->lcnt[gen & 3], k);
     if (work_dst && sh.wsum) atomic_add64(work_dst, sh.wsum);
@@ -328,7 +332,7 @@ static __device__ void phase_end(const Dev &D, Shared &sh, int gen, long long wo
         set_err(D, MF_ERR_INTERNAL, 11);
     }
   }
-  int *lq = sh.lq[gen % 3];
+  int *lq = sh.lq[gen % 3] + sh.lq0;
   for (int i = threadIdx.x; i < sh.lk; i += blockDim.x) lq[i] = sh.qbuf[i];
 }
 
@@ -1214,28 +1218,58 @@ __device__ void relabel_phase(const Dev &D, Shared &sh, int r, int gen, long lon
   for (int off = 0; off < sw.items; off += blockDim.x) {
     int x = -1;
     int v = -1, beg = 0, deg = 0, cls = 0, cap_v = 0, k = -1;
-    if (sweep_item(sw, sweep_pos(off, sw.items), x) == 1) {
+    int newl = INT_MAX, open = 0;
+    const int item = sweep_pos(off, sw.items);
+    if (sweep_item(sw, item, x) == 1) {
       v = x;
       const int dv = __ldcg(lab_ptr(D, v, R.p));
+      const longlong2 ea = load_ea(D, v);
       const int2 vi = vinst_of<MULTI>(D, v);
       cap_v = vi.x;
       k = vi.y;
-      // Section 3 step 4 for this vertex: the excess it received this round joins its excess now
-      const long long ex_own = __ldcg(exc_ptr(D, v));
-      const long long ad = dv >= cap_v ? 0 : take_added(D, v);
-      if (ad) *exc_ptr(D, v) = ex_own + ad;
+      // a kept entry's row and heads, loaded before the push pass: its arcs and their heads' labels in the
+      // same round trip as its own record
+      const bool pre = item < (int)blockDim.x && sh.pv[item] == x && sh.pdeg[item] <= D.bin_thread;
+      if (pre) {
+        beg = sh.pbeg[item];
+        deg = sh.pdeg[item];
+        int rs[KT], lw[KT];
+#pragma unroll
+        for (int i = 0; i < KT; i++) {
+          rs[i] = 0;
+          lw[i] = 0;
+          if (i < deg) {
+            rs[i] = __ldcg(&D.rr[MF_SLOT(D, beg + i)]).x;
+            lw[i] = __ldcg(lab_ptr(D, sh.phead[i][item], R.p));
+          }
+        }
+#pragma unroll
+        for (int i = 0; i < KT; i++)
+          if (rs[i] > 0) {
+            newl = min(newl, lw[i] + 1);
+            open++;
+          }
+      }
+      // Section 3 step 4 for this vertex: the excess it received this round joins its excess now (nobody
+      // adds to either until the next round)
+      if (dv < cap_v && ea.y) {
+        *exc_ptr(D, v) = ea.x + ea.y;
+        *add_ptr(D, v) = 0;
+      }
       if (dv >= cap_v) {
         v = -1;  // retired in the push step
-      } else if (ex_own == 0) {
+      } else if (ea.x == 0) {
         *lab_ptr(D, v, R.p ^ 1) = dv;
         v = -1;
+      } else if (pre) {
+        st.scans_dis += deg;
+        st.scans_res += open;
       } else {
         beg = __ldg(&D.row[MF_ROW(D, v)]);
         deg = __ldg(&D.row[MF_ROW(D, v + 1)]) - beg;
         cls = deg <= D.bin_thread ? 1 : (deg <= D.bin_warp ? 2 : 3);
       }
     }
-    int newl = INT_MAX;
     for (bool any = D.cta_vertices && __syncthreads_or(cls == 3); any;) {  // CTA per vertex
       if (threadIdx.x == 0) sh.pick = -1;
       __syncthreads();
@@ -1307,7 +1341,7 @@ __device__ void relabel_phase(const Dev &D, Shared &sh, int r, int gen, long lon
     __syncwarp();
     if (MULTI && D.inst_relabel) inst_add_work(D, k, wt, R.rnd);
   }
-  phase_end(D, sh, R.next, work, &D.ctl->work[rnd % 3]);
+  phase_end(D, sh, R.next, work, &D.ctl->work[rnd % 3], true);  // (the push pass staged what received excess)
 }
 
 // ------------------------------------------------------------------ BFS
@@ -2006,7 +2040,7 @@ __device__ bool run_phase(const Dev &D, Shared &sh, const int *sinks, const int 
     if (!grid_sync(D, sh, 4, D.simple ? PF_NONE : PF_ROUND, gen + 1, gen)) return false;
     if (D.simple) {
       relabel_phase<MULTI>(D, sh, r, gen, rnd, st);
-      if (!grid_sync(D, sh, 4)) return false;
+      if (!grid_sync(D, sh, 4, PF_ROUND, gen + 1, gen)) return false;
     }
     if (timer) {
       const unsigned long long t3 = gtimer();
@@ -2248,7 +2282,7 @@ __device__ bool run_union(const Dev &D, Shared &sh, int &r, int &gen, long long 
     if (!grid_sync(D, sh, 4, D.simple ? PF_NONE : PF_ROUND, gen + 1, gen)) return false;
     if (D.simple) {
       relabel_phase<true>(D, sh, r, gen, rnd, st);
-      if (!grid_sync(D, sh, 4)) return false;
+      if (!grid_sync(D, sh, 4, PF_ROUND, gen + 1, gen)) return false;
     }
     if (timer) {
       const unsigned long long t3 = gtimer();
