@@ -344,6 +344,7 @@ Dev make_dev(const mf_graph *g) {
   D.simple = g->opt.simple_rounds ? 1 : 0;
   D.cta_vertices = g->max_degree > (long long)g->opt.bin_warp ? 1 : 0;
   D.keep_local = keep_local_limit(g->opt, g->max_degree, g->block);
+  D.hub_runs = hub_runs_apply(g->n, g->m, g->max_degree) ? 1 : 0;
   D.bfs_hops = D.keep_local > 0 ? g->opt.bfs_hops : 1;
   D.gap_every = (g->ninst == 1 && !D.simple && g->hist) ? g->opt.gap_every : 0;
   D.bfs_pull = g->opt.bfs_pull;

@@ -50,6 +50,7 @@ struct Ctl {
   int cut_pending;        // unions: a relabel ended the flow phase of some instances (they need their cut)
   int done_cnt;           // unions: instances whose results are written
   int qhead[4], qtail[4], qidle[4];  // lattice solves: tickets taken, entries made and warps waiting, by phase % 4
+  int hub_runs[2];        // single graphs: runs of arcs of the hubs of a BFS level, by list generation % 2
   int runs;               // unions: runs of arcs of the seeds a BFS does not queue
   long long bad_index;    // builds with MF_CHECK_BOUNDS: the first gather index found outside its array
 };
@@ -176,6 +177,8 @@ struct Dev {
   int simple;              // 1: the simple synchronous rounds of Section 3 (push pass, then one relabel)
   int cta_vertices;        // 0: no vertex other than a source or sink has more than bin_warp slots, so no
                            //    discharge needs a whole CTA (the CTA-wide check is skipped)
+  int hub_runs;            // 1: BFS levels share the arcs of hubs among all CTAs (some vertex has enough arcs, and the
+                           //    lists can hold the runs)
   int keep_local;          // a CTA that stages at most this many entries of a list generation keeps them in
                            // its shared memory for the phase that consumes the generation instead of
                            // appending them to the list in global memory (0: always append). Set only when

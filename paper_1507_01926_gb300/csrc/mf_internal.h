@@ -90,6 +90,7 @@ int run_kernel(mf_graph *g, Dev &D, cudaStream_t st);
 int launch_kernel(mf_graph *g, Dev &D, cudaStream_t st);
 int finish_kernel(mf_graph *g);
 int keep_local_limit(const mf_options &o, long long max_degree, int block_threads);
+bool hub_runs_apply(long long n, long long m, long long max_degree);
 int solver_variants();
 int solver_variant_max_threads(int variant);
 int solver_variant_max_bin_thread(int variant);

@@ -51,6 +51,10 @@ int keep_local_limit(const mf_options &o, long long max_degree, int block_thread
   return k < block_threads ? k : block_threads;  // block_threads <= MAX_BLOCK
 }
 
+bool hub_runs_apply(long long n, long long m, long long max_degree) {
+  return max_degree > HUB_MIN && 2 * (m / RUN_ARCS + m / HUB_MIN) <= n;
+}
+
 int solver_occupancy(int block_threads, int *blocks_per_sm, int variant, bool multi) {
   if (variant < 0 || variant >= NUM_VARIANTS) return -1;
   const void *fn = kernel_fn(variant, multi);

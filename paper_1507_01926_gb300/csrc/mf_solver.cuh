@@ -1493,12 +1493,48 @@ __device__ __forceinline__ void bfs_thread(const Dev &D, Shared &sh, int beg, in
     if (bfs_won(old[i], c)) qpush(D, sh, next, w[i]);
 }
 
+// Seeds of a union with more arcs than a CTA has threads (the terminals of its
+// images: one CTA walked the 115,000 arcs of a 14-frame video's sink in 0.45 ms,
+// in every relabel) are not queued: their arcs are cut into runs that the CTAs
+// share in the first level. The runs {first, end} are kept in the list of
+// generation gen + 2, which is not in use then; unions whose lists could not hold
+// them (few vertices with very many arcs) queue all seeds.
+constexpr int RUN_ARCS = 1024;
+
+__device__ __forceinline__ bool runs_fit(const Dev &D) {
+  return 2LL * ((long long)D.m / RUN_ARCS + 2LL * D.ninst) <= D.n;
+}
+
+// Vertices above this are shared by the grid in a BFS level of a single graph: the
+// extra grid barrier of every level (2-3 us) is paid back where a CTA would walk
+// 16 or more runs alone (about 5 us each).
+constexpr int HUB_MIN = 16 * RUN_ARCS;
+
+// Adds the runs of the arcs [b, e) to the list `to`, counted by *count.
+__device__ __forceinline__ void put_runs(const Dev &D, int *to, int *count, int b, int e) {
+  int at = atomicAdd(count, (e - b + RUN_ARCS - 1) / RUN_ARCS);
+  for (; b < e; at++) {
+    const int n = min(e - b, RUN_ARCS);
+    to[2 * at] = b;
+    to[2 * at + 1] = b + n;
+    b += n;
+  }
+}
+
 // One BFS level: expands the list of generation gen into generation gen + 1,
 // then (D.bfs_hops > 1) up to bfs_hops - 1 more levels of the vertices this
 // CTA reached itself, while they fit one per thread.
+//
+// In a single graph with D.hub_runs, vertices with more than HUB_MIN arcs are not
+// walked by the CTA that finds them on the list: their arcs are cut into runs of
+// RUN_ARCS that all CTAs share after one more grid barrier (their list of
+// generation gen + 2 holds the runs; such graphs have no CTA-local levels, so
+// every vertex of the level has the same label). On an R-MAT graph of scale 22
+// (4.2 million vertices, 67 million arcs) one hub kept a level waiting for 2-3 ms:
+// solve kernel 83 -> 77 ms.
 template <int KTD, bool MULTI>
-__device__ void bfs_level(const Dev &D, Shared &sh, int gen, bool reverse, TStat &st, const Ends &E, const Final &one,
-                          int runs) {
+__device__ bool bfs_level(const Dev &D, Shared &sh, int gen, int depth, bool reverse, TStat &st, const Ends &E,
+                          const Final &one, int runs, int where) {
   const int next = gen + 1;
   if (MULTI)  // level 0 of the union's seeds with many arcs
     for (int i = blockIdx.x; i < runs; i += gridDim.x) {
@@ -1511,6 +1547,7 @@ __device__ void bfs_level(const Dev &D, Shared &sh, int gen, bool reverse, TStat
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     D.ctl->cnt[(gen + 2) & 3] = 0;
     D.ctl->lcnt[(gen + 2) & 3] = 0;
+    D.ctl->hub_runs[(gen + 1) & 1] = 0;
   }
   const int lane = threadIdx.x & 31;
   for (int off = 0; off < sw.items; off += blockDim.x) {
@@ -1531,6 +1568,10 @@ __device__ void bfs_level(const Dev &D, Shared &sh, int gen, bool reverse, TStat
         deg = __ldg(&D.row[MF_ROW(D, v + 1)]) - beg;
       }
       cls = deg <= KTD ? 1 : (deg <= D.bin_warp ? 2 : 3);
+      if (!MULTI && D.hub_runs && deg > HUB_MIN) {
+        put_runs(D, list_of(D, gen + 2), &D.ctl->hub_runs[gen & 1], beg, beg + deg);
+        cls = 0;
+      }
       st.scans_bfs += deg;
       st.visits_bfs++;
     }
@@ -1570,6 +1611,14 @@ __device__ void bfs_level(const Dev &D, Shared &sh, int gen, bool reverse, TStat
     if (cls == 1) bfs_thread<KTD>(D, sh, beg, deg, l, reverse, next, pre ? item : -1, F);
     __syncwarp();
   }
+  if (!MULTI && D.hub_runs) {
+    if (!grid_sync(D, sh, where)) return false;
+    const int n = __ldcg(&D.ctl->hub_runs[gen & 1]);
+    for (int i = blockIdx.x; i < n; i += gridDim.x) {
+      const int a = __ldcg(&list_of(D, gen + 2)[2 * i]), e = __ldcg(&list_of(D, gen + 2)[2 * i + 1]);
+      bfs_arcs(D, sh, a + (int)threadIdx.x, e, blockDim.x, depth + 1, reverse, next, one);
+    }
+  }
   // more levels inside the CTA (only on graphs whose vertices are all
   // thread-sized; staged entries are taken out of the staging buffer)
   for (int hop = 1; hop < D.bfs_hops; hop++) {
@@ -1599,6 +1648,7 @@ __device__ void bfs_level(const Dev &D, Shared &sh, int gen, bool reverse, TStat
     }
   }
   phase_end(D, sh, next, 0, nullptr);
+  return true;
 }
 
 // One bottom-up level (direction-optimizing BFS, Beamer, Asanovic and Patterson
@@ -1615,6 +1665,7 @@ static __device__ void bfs_pull_level(const Dev &D, Shared &sh, int gen, int dep
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     D.ctl->cnt[(gen + 2) & 3] = 0;
     D.ctl->lcnt[(gen + 2) & 3] = 0;
+    D.ctl->hub_runs[(gen + 1) & 1] = 0;
   }
   const int lane = threadIdx.x & 31;
   for_covered(D, S, [&](int wv, bool valid) {
@@ -1689,18 +1740,6 @@ __device__ __forceinline__ void level_done(const Dev &D, unsigned long long t0, 
   D.ctl->t_lwait += t2 - t1;
 }
 
-// Seeds of a union with more arcs than a CTA has threads (the terminals of its
-// images: one CTA walked the 115,000 arcs of a 14-frame video's sink in 0.45 ms,
-// in every relabel) are not queued: their arcs are cut into runs that the CTAs
-// share in the first level. The runs {first, end} are kept in the list of
-// generation gen + 2, which is not in use then; unions whose lists could not hold
-// them (few vertices with very many arcs) queue all seeds.
-constexpr int RUN_ARCS = 1024;
-
-__device__ __forceinline__ bool runs_fit(const Dev &D) {
-  return 2LL * ((long long)D.m / RUN_ARCS + 2LL * D.ninst) <= D.n;
-}
-
 // Level 0 of a BFS from one seed with many arcs (slots [b, e)), the seed
 // labelled 0 and not queued (generation gen is empty): the whole grid offers
 // label 1 along its arcs, one arc per thread, into generation gen + 1. Ends
@@ -1744,6 +1783,7 @@ __device__ bool bfs(const Dev &D, Shared &sh, const int *seeds, const int *block
     D.ctl->cnt[(gen + 2) & 3] = 0;
     D.ctl->lcnt[(gen + 2) & 3] = 0;
     D.ctl->runs = 0;
+    D.ctl->hub_runs[0] = D.ctl->hub_runs[1] = 0;
   }
   const bool in_runs = MULTI && runs_fit(D);
   for_covered(D, S, [&](int v, bool valid) {
@@ -1784,11 +1824,7 @@ __device__ bool bfs(const Dev &D, Shared &sh, const int *seeds, const int *block
       const int b = __ldg(&D.row[MF_ROW(D, v)]), e = __ldg(&D.row[MF_ROW(D, v + 1)]);
       if (e - b > (int)blockDim.x) {
         queued = false;
-        int at = atomicAdd(&D.ctl->runs, (e - b + RUN_ARCS - 1) / RUN_ARCS);
-        for (int a = b; a < e; a += RUN_ARCS, at++) {
-          list_of(D, gen + 3)[2 * at] = a;  // gen + 2 of the level loop's first generation
-          list_of(D, gen + 3)[2 * at + 1] = min(e - a, RUN_ARCS) + a;
-        }
+        put_runs(D, list_of(D, gen + 3), &D.ctl->runs, b, e);  // gen + 2 of the level loop's first generation
         st.visits_bfs++;
       }
     }
@@ -1818,8 +1854,8 @@ __device__ bool bfs(const Dev &D, Shared &sh, const int *seeds, const int *block
     // BFS, where every frontier vertex carries the label `depth`)
     if (D.bfs_pull > 0 && D.bfs_hops == 1 && fcount * D.bfs_pull > D.n && runs == 0)
       bfs_pull_level(D, sh, gen, depth, reverse, st, S);
-    else
-      bfs_level<KTD, MULTI>(D, sh, gen, reverse, st, Ends{seeds, blockers}, F, runs);
+    else if (!bfs_level<KTD, MULTI>(D, sh, gen, depth, reverse, st, Ends{seeds, blockers}, F, runs, where))
+      return false;
     runs = 0;
     const unsigned long long t1 = timer ? gtimer() : 0;
     if (!grid_sync(D, sh, where, PF_LEVEL, gen + 1)) return false;
