@@ -18,11 +18,12 @@
 // registers; a visit loads it, runs several rounds on it without leaving the SM,
 // and writes it back. Excess crosses a whole tile per visit, and a BFS label too.
 //
-//  * Inside a tile a cell pushes along residual arcs to lower labels, and with
-//    excess left relabels (one above the least residual neighbour) and pushes
-//    once more. Cells of a tile do so at the same time on labels that may be one
-//    round old, as in the paper's synchronous rounds, and without its win rule: a
-//    label may then rise past the distance, which costs detours, not correctness.
+//  * Inside a tile a cell pushes along residual arcs to lower labels and relabels
+//    (one above the least residual neighbour): in 2D after the push, with excess
+//    left, and pushes once more; in 3D before it, when no such arc is there. Cells
+//    of a tile do so at the same time on labels that may be one round old, as in
+//    the paper's synchronous rounds, and without its win rule: a label may then
+//    rise past the distance, which costs detours, not correctness.
 //  * A push over a tile face uses the neighbour's label as it was when the tile
 //    was loaded, takes the residual from the pusher's side at once and adds the
 //    amount to the receiver's inbox; it joins the receiver's excess and its side

@@ -4,9 +4,14 @@
 // active in a round, three or four of them, so a round is a short dependent chain
 // on a few lanes. With a CTA per tile, nearly every warp has one active lane and
 // all of them wait at the CTA barriers (a round took 1.3 us, four tiles per SM); a
-// warp per tile runs the same round in 0.6-0.9 us, eight tiles per SM. A visit is
-// about 17 us: 4 us to load 25 KB and take in the inboxes, ten rounds, 2.5 us to
-// write the touched cells back and hand on to the neighbours.
+// warp per tile runs the same round in 0.6 us, eight tiles per SM. A visit is
+// about 16 us: 4 us to load 25 KB and take in the inboxes, ten rounds, 2.5 us to
+// write the touched cells back and hand on to the neighbours. A scheduler issues
+// an instruction every 8 cycles; of a warp's time a quarter is waiting for a tile
+// (97x80x61 has fewer active tiles than the GPU has warps), a quarter loads, a
+// third the dependent instructions and branches of the rounds.
+// Measured, solve of 97x80x61 / 256x256x128: list solver 96 / 870 ms, a CTA per
+// tile in sweeps 30 / 750 ms, this 30 / 415 ms.
 #include "mf_lattice.cuh"
 #include "mf_internal.h"
 
@@ -270,13 +275,17 @@ __device__ __forceinline__ void push_out(const Dev &D, const LTile<DIM> &w, int 
   atomicAdd(&D.lat.inbox[(size_t)w.nt[j] * G::NH + (j ^ 1) * G::FS + G::face(j, u)], a);
 }
 
-// A round over the warp's list (n cells), 32 at a time, a lane per cell: every lane reads its cell and its neighbours' labels, pushes along the arcs
-// that lead to lower labels and, with excess left, relabels and pushes once more.
-// Returns the number of cells on the next list. Residuals change by atomics, as
-// a relabeled cell and its neighbour may push over the same pair at once (then
-// its labels are not valid in the sense of Section 2.1, which costs detours, not
-// correctness). Nothing waits for an atomic's result: what a cell received and
-// whether it is active next are sums and bits read in the next round.
+// A round over the warp's list (n cells), 32 at a time, a lane per cell: every lane
+// reads its cell and its neighbours' labels, relabels first if no residual arc
+// leads to a lower label, and pushes along those that do. Excess left after that
+// waits for the next round. (Pushing, relabeling and pushing again in one round
+// took 5-10% longer on 97x80x61 and 256x256x128: fewer rounds, but the second pass
+// ran in nearly all of them.) Returns the number of cells on the next list.
+// Residuals change by atomics, as a relabeled cell and its neighbour may push over
+// the same pair at once (then its labels are not valid in the sense of Section 2.1,
+// which costs detours, not correctness). Nothing waits for an atomic's result: what
+// a cell received and whether it is active next are sums and bits read in the next
+// round.
 template <int DIM>
 __device__ __forceinline__ int push_round(const Dev &D, LTile<DIM> &w, int t, int n, unsigned char *ret, unsigned &out,
                                           unsigned &touched, LStat &st) {
@@ -313,39 +322,33 @@ __device__ __forceinline__ int push_round(const Dev &D, LTile<DIM> &w, int t, in
       }
     }
     __syncwarp();  // every lane has read its cell
-    int lab = du;
-#pragma unroll 1
-    for (int pass = 0;; pass++) {
-      int m = LINF;  // (excess is left only where the drain is used up)
+    int m = LINF;
 #pragma unroll
-      for (int j = 0; j < G::ND; j++) {
-        const int a = dl[j] < lab ? min(r[j], left) : 0;
-        left -= a;
-        r[j] -= a;
-        if (r[j] > 0) m = min(m, dl[j]);
-        if (a > 0) {
-          st.pushes++;
-          atomicAdd(&w.r[j][u], -a);
-          if (G::inside(j, u)) {
-            const int x = u + G::step(j);
-            atomicAdd(&w.r[j ^ 1][x], a);
-            give<DIM>(w, x, a);
-            mark<DIM>(w, x);
-          } else {
-            push_out<DIM>(D, w, j, u, a);
-            out |= 1u << j;
-          }
+    for (int j = 0; j < G::ND; j++) m = min(m, r[j] > 0 ? dl[j] : LINF);
+    int lab = du;
+    if (left > 0 && m >= lab) {
+      lab = min(m + 1, LINF);
+      st.relabels++;
+    }
+    const int can = lab < cap ? left : 0;
+    e += left - can;
+    left = can;
+#pragma unroll
+    for (int j = 0; j < G::ND; j++) {
+      const int a = dl[j] < lab ? min(r[j], left) : 0;
+      left -= a;
+      if (a > 0) {
+        st.pushes++;
+        atomicAdd(&w.r[j][u], -a);
+        if (G::inside(j, u)) {
+          const int x = u + G::step(j);
+          atomicAdd(&w.r[j ^ 1][x], a);
+          give<DIM>(w, x, a);
+          mark<DIM>(w, x);
+        } else {
+          push_out<DIM>(D, w, j, u, a);
+          out |= 1u << j;
         }
-      }
-      const bool up = left > 0 && m + 1 > lab;
-      if (up) {
-        lab = min(m + 1, LINF);
-        st.relabels++;
-      }
-      if (pass || !__any_sync(LFULL, up && lab < cap)) break;
-      if (lab >= cap) {  // out of the second pass
-        e += left;
-        left = 0;
       }
     }
     if (on) {
