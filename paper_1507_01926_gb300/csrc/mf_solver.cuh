@@ -60,6 +60,8 @@ constexpr unsigned FULL = 0xffffffffu;
 constexpr int KT = 8;           // largest degree handled by one thread (register-cached arcs)
 constexpr int MAX_BLOCK = 512;  // largest CTA
 constexpr int MAX_WARPS = MAX_BLOCK / 32;
+// Arcs each thread of a CTA takes per chunk of a CTA-sized vertex: in a discharge, in a BFS.
+constexpr int DIS_ARCS = 2, HUB_ARCS = 4;
 
 // ------------------------------------------------------------------ helpers
 
@@ -221,7 +223,6 @@ struct Shared {
   unsigned long long bars;  // grid barriers passed by this CTA
   Snap snap;
   int pick;
-  int flag;
   int qn;                   // staged appends (may exceed QCAP; the excess went straight to the list)
   int qbase;
   int qk;                   // staged entries to publish to the list in global memory
@@ -229,7 +230,7 @@ struct Shared {
   int lq0;                  // entries of the generation kept before
   long long wsum;
   int imin[MAX_WARPS];
-  long long lsum[4 * MAX_WARPS];  // HUB_ARCS sub-chunks of a CTA-sized vertex
+  long long lsum[DIS_ARCS * MAX_WARPS];  // per sub-chunk of a CTA-sized vertex and warp
   int lqn[3];               // kept entries of list generation g, in lq[g % 3]
   int qbuf[QCAP];
   int qrow[MAX_BLOCK];      // BFS staging: row[v] of qbuf[i] (i < MAX_BLOCK) when known (qdeg[i] >= 0)
@@ -961,17 +962,19 @@ static __device__ void discharge_warp(const Dev &D, Shared &sh, const RoundCtx &
   __syncwarp();
 }
 
-// Arcs each thread of a CTA takes per chunk of a CTA-sized vertex.
-constexpr int HUB_ARCS = 4;
-
-// One CTA (all threads call), arcs in chunks of HUB_ARCS * blockDim: thread t
-// holds arcs t, t + blockDim, ... of the chunk, so that loads are coalesced and
-// the dependent loads of HUB_ARCS arcs are in flight together, the prefix sum
-// over the chunk (arc order) needs the same CTA barriers as one arc per thread
-// would, and the next chunk's heads and residuals are loaded meanwhile (they can
-// only grow until then, by pushes into v). What is left is the latency of the
-// labels, random sectors, once per chunk. On an R-MAT graph of scale 22: solve
-// kernel 77 -> 69-74 ms.
+// One CTA (all threads call), arcs in chunks of DIS_ARCS * blockDim: thread t
+// holds arcs t, t + blockDim, ... of the chunk, so that loads are coalesced. What
+// bounds it is the latency of a chunk, as one hub with half a million arcs is a
+// round of its own: while a chunk is worked on, the labels of the next one and the
+// heads and residuals of the one after that are on their way (labels do not change
+// in a round, and residuals read early can only have grown, by pushes into v). A
+// chunk without a pushable arc, the usual one where the pass is for a relabel,
+// costs one CTA barrier; the others also a prefix sum over the chunk (arc order)
+// and a second one. On an R-MAT graph of scale 22 (67 million arcs), solve kernel
+// with kernel variant 1 (80 registers) / 0 (128): 70 / 66 ms with the next heads
+// and residuals loaded early, three barriers and 4 arcs per thread; 70 / 50 ms with
+// the labels early too and one barrier where nothing is pushed (16 more registers,
+// which variant 1 spills); 57 / 48 ms with 2 arcs per thread.
 static __device__ void discharge_block(const Dev &D, const RoundCtx &R, int v, int dv, int cap_v, TStat &st,
                                 long long &work, Shared &sh) {
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
@@ -984,64 +987,74 @@ static __device__ void discharge_block(const Dev &D, const RoundCtx &R, int v, i
   int dp = dv;
   long long to_sink = 0;
   int sink = -1;
+  const int chunk = DIS_ARCS * (int)blockDim.x;
+  auto fetch = [&](long long c, int (&hw)[DIS_ARCS], int (&hr)[DIS_ARCS]) {
+#pragma unroll
+    for (int u = 0; u < DIS_ARCS; u++) {
+      const long long i = c + u * (int)blockDim.x + (int)threadIdx.x;
+      hw[u] = 0;
+      hr[u] = 0;
+      if (i < deg) {
+        hw[u] = __ldg(&D.head[MF_SLOT(D, beg + i)]);
+        hr[u] = __ldcg(&D.rr[MF_SLOT(D, beg + i)]).x;
+      }
+    }
+  };
+  auto labels = [&](const int (&hw)[DIS_ARCS], const int (&hr)[DIS_ARCS], int2 (&x)[DIS_ARCS]) {
+#pragma unroll
+    for (int u = 0; u < DIS_ARCS; u++) x[u] = hr[u] > 0 ? load_slot(D, R.p, hw[u]) : make_int2(0, 0);
+  };
   for (;;) {
     int newl = cap_v;
-    int skipped = 0;
-    int nw4[HUB_ARCS], nrs[HUB_ARCS];  // heads and residuals of the chunk that comes next
-    auto fetch = [&](long long c) {
-#pragma unroll
-      for (int u = 0; u < HUB_ARCS; u++) {
-        const long long i = c + u * (int)blockDim.x + (int)threadIdx.x;
-        nw4[u] = 0;
-        nrs[u] = 0;
-        if (i < deg) {
-          nw4[u] = __ldg(&D.head[MF_SLOT(D, beg + i)]);
-          nrs[u] = __ldcg(&D.rr[MF_SLOT(D, beg + i)]).x;
-        }
-      }
-    };
-    fetch(0);
-    for (long long c = 0; c < deg && ex > 0; c += HUB_ARCS * (int)blockDim.x) {
-      int w[HUB_ARCS], rs[HUB_ARCS], dw[HUB_ARCS];
+    int skipped = 0;  // this thread's arcs
+    int w1[DIS_ARCS], r1[DIS_ARCS], w2[DIS_ARCS], r2[DIS_ARCS];  // heads and residuals of the next two chunks
+    int2 x1[DIS_ARCS];                                           // labels and stamps of the next chunk's heads
+    fetch(0, w1, r1);
+    fetch(chunk, w2, r2);
+    labels(w1, r1, x1);
+    for (long long c = 0; c < deg && ex > 0; c += chunk) {
+      int w[DIS_ARCS], rs[DIS_ARCS], dw[DIS_ARCS];
       unsigned wact = 0, push = 0, skip = 0;  // bit u: w in the working set, arc pushable, arc skipped
 #pragma unroll
-      for (int u = 0; u < HUB_ARCS; u++) {
-        w[u] = nw4[u];
-        rs[u] = nrs[u];
-        dw[u] = 0;
+      for (int u = 0; u < DIS_ARCS; u++) {
+        w[u] = w1[u];
+        rs[u] = r1[u];
+        dw[u] = x1[u].x;
+        wact |= (unsigned)(x1[u].y == R.r) << u;
+        w1[u] = w2[u];
+        r1[u] = r2[u];
         st.scans_dis += c + u * (int)blockDim.x + (int)threadIdx.x < deg;
+        st.scans_res += rs[u] > 0;
       }
+      labels(w1, r1, x1);
+      fetch(c + 2 * chunk, w2, r2);
 #pragma unroll
-      for (int u = 0; u < HUB_ARCS; u++)
-        if (rs[u] > 0) {
-          const int2 x = load_slot(D, R.p, w[u]);
-          dw[u] = x.x;
-          if (x.y == R.r) wact |= 1u << u;
-          st.scans_res++;
-        }
-      fetch(c + HUB_ARCS * (int)blockDim.x);  // in flight while this chunk's labels come and its pushes go
-#pragma unroll
-      for (int u = 0; u < HUB_ARCS; u++)
+      for (int u = 0; u < DIS_ARCS; u++)
         if (rs[u] > 0 && dp == dw[u] + 1) {
           if (!D.simple && ((wact >> u) & 1u) && !wins(dv, dw[u], v, w[u]))
             skip |= 1u << u;
           else
             push |= 1u << u;
         }
-      __syncthreads();  // previous chunk finished reading sh
-      if (threadIdx.x == 0) sh.flag = 0;
-      long long incl[HUB_ARCS];
+      skipped |= (int)skip;
+      const bool pushes = __syncthreads_or((int)push);  // (and the previous chunk's sums are read)
+      if (!pushes) {
 #pragma unroll
-      for (int u = 0; u < HUB_ARCS; u++) {
+        for (int u = 0; u < DIS_ARCS; u++)
+          if (!((skip >> u) & 1u) && rs[u] > 0 && dw[u] >= dp) newl = min(newl, dw[u] + 1);
+        continue;
+      }
+      long long incl[DIS_ARCS];
+#pragma unroll
+      for (int u = 0; u < DIS_ARCS; u++) {
         const bool p = (push >> u) & 1u;
         incl[u] = __ballot_sync(FULL, p) ? warp_incl_scan(p ? (long long)rs[u] : 0, lane) : 0;
         if (lane == 31) sh.lsum[u * MAX_WARPS + wid] = incl[u];
       }
       __syncthreads();
-      if (skip) sh.flag = 1;
       long long base = 0;  // pushable residuals of the arcs before sub-chunk u
 #pragma unroll
-      for (int u = 0; u < HUB_ARCS; u++) {
+      for (int u = 0; u < DIS_ARCS; u++) {
         long long wbase = base;
         for (int k = 0; k < nw; k++) {
           const long long x = sh.lsum[u * MAX_WARPS + k];
@@ -1068,10 +1081,9 @@ static __device__ void discharge_block(const Dev &D, const RoundCtx &R, int v, i
         if (found) qpush(D, sh, R.next, w[u]);
         if (!((skip >> u) & 1u) && rs[u] > 0 && dw[u] >= dp) newl = min(newl, dw[u] + 1);
       }
-      __syncthreads();
-      skipped |= sh.flag;
       ex = base >= ex ? 0 : ex - base;
     }
+    skipped = __syncthreads_or(skipped);
     // block min of newl
     int wm = warp_min(newl);
     __syncthreads();
