@@ -42,7 +42,8 @@ __global__ void k_lat_strides(int n, const int *row, const int *head, Lat L, int
 
 // Sets *bad when some arc does not join neighbouring cells of the X x Y x Z box
 // (or a cell and a terminal), a cell has two slots in one direction or to one
-// terminal, or s and t are joined directly.
+// terminal, or s and t are joined directly, to each other or to themselves (the
+// outputs of terminals are written from the cells' slots).
 __global__ void k_lat_check(int n, const int *row, const int *head, Lat L, int *bad) {
   bool f = false;
   const int A = L.X, B = L.X * L.Y;
@@ -73,8 +74,11 @@ __global__ void k_lat_check(int n, const int *row, const int *head, Lat L, int *
     }
   }
   const int tid = blockIdx.x * blockDim.x + threadIdx.x;
-  for (int a = row[L.s] + tid; a < row[L.s + 1]; a += gridDim.x * blockDim.x)
-    if (head[a] == L.t || head[a] == L.s) f = true;
+  for (int k = 0; k < 2; k++) {
+    const int v = k ? L.t : L.s;
+    for (long long a = (long long)row[v] + tid; a < row[v + 1]; a += gridDim.x * blockDim.x)
+      if (head[a] == L.t || head[a] == L.s) f = true;
+  }
   if (__any_sync(LFULL, f) && (threadIdx.x & 31) == 0) atomicOr(bad, 1);
 }
 

@@ -1,0 +1,76 @@
+"""Which solver a call runs and what it leaves behind, for single 2D and 3D grids (the lattice solvers) and graphs
+that are nearly such grids (the list solver). A lattice solve counts no rounds by size, a list solve does."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_1507_01926_gb300 import inputs as I
+
+pytestmark = pytest.mark.gpu
+
+
+def grid(dims, seed):
+    """A lattice whose cells all have an arc from s or to t (side lengths from the slowest axis to the fastest)."""
+    rng = np.random.default_rng(seed)
+    idx = np.arange(int(np.prod(dims))).reshape(dims)
+    u = np.concatenate([np.take(idx, np.arange(d - 1), axis=k).ravel() for k, d in enumerate(dims)])
+    v = np.concatenate([np.take(idx, np.arange(1, d), axis=k).ravel() for k, d in enumerate(dims)])
+    n = idx.size
+    src = rng.random(n) < 0.5
+    cells = np.arange(n)
+    tail = np.concatenate([u, v, np.where(src, n, cells)])
+    head = np.concatenate([v, u, np.where(src, cells, n + 1)])
+    cap = np.concatenate([rng.integers(1, 101, 2 * u.size), rng.integers(1, 201, n)])
+    return I.Instance(n + 2, n, n + 1, tail.astype(np.int32), head.astype(np.int32), cap.astype(np.int32), f"grid_{dims}")
+
+
+def on_lattice(stats):
+    return stats["rounds"] > 0 and not any(stats["rounds_by_size"])
+
+
+def on_lists(stats):
+    return any(stats["rounds_by_size"])
+
+
+def add_self_loop(csr, v):
+    """The CSR with one more slot pair v -> v at the end of v's row."""
+    at = int(csr.row_offsets[v + 1])
+    row = csr.row_offsets.copy()
+    row[v + 1:] += 2
+    rev = csr.rev + 2 * (csr.rev >= at)
+    return (row, np.insert(csr.head, at, [v, v]).astype(np.int32), np.insert(csr.cap, at, [3, 4]).astype(np.int32),
+            np.insert(rev, at, [at + 1, at]).astype(np.int64), at)
+
+
+DIMS = [(20, 33), (9, 10, 11)]
+
+
+@pytest.mark.parametrize("dims", DIMS)
+@pytest.mark.parametrize("where", ["s", "t", "cell"])
+def test_self_loops_have_their_flow_written(gpu, dims, where):
+    """A raw CSR may hold slot pairs from a vertex to itself (mf_build_csr drops them): the graph is no lattice, and
+    every slot of the flow output is written."""
+    import torch
+
+    g = grid(dims, 1)
+    csr = gpu.build_csr(g.n, g.tail, g.head, g.cap)
+    row, head, cap, rev, at = add_self_loop(csr, {"s": g.s, "t": g.t, "cell": 7}[where])
+    dev = torch.device("cuda", 0)
+    st = torch.cuda.Stream()
+    arrays = [torch.from_numpy(a).to(dev) for a in (row, head, cap, rev)]
+    val = torch.zeros(1, dtype=torch.int64, device=dev)
+    flow = torch.full((head.size,), -7, dtype=torch.int32, device=dev)
+    cut = torch.zeros((g.n + 31) // 32, dtype=torch.int32, device=dev)
+    torch.cuda.synchronize()
+    G = gpu.Graph.from_device(g.n, *arrays, g.s, g.t, stream=st)
+    try:
+        G.solve_device(val, flow, cut, stream=st)
+        stats = G.stats()
+    finally:
+        G.close()
+    ref = oracle.maxflow(g.n, g.s, g.t, g.tail, g.head, g.cap, want_flow=False)
+    f = flow.cpu().numpy()
+    assert int(val.item()) == ref["value"]
+    assert np.array_equal(gpu.cut_bits_to_bool(cut.cpu().numpy().view(np.uint32), g.n), ref["cut"])
+    assert f[at] == 0 and f[at + 1] == 0 and f.min() >= 0
+    assert on_lists(stats)
