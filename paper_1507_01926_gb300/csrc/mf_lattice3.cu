@@ -13,6 +13,7 @@
 // Measured, solve of 97x80x61 / 256x256x128: list solver 96 / 870 ms, a CTA per
 // tile in sweeps 30 / 750 ms, this 30 / 415 ms.
 #include "mf_lattice.cuh"
+#include "mf_tile_queue.cuh"
 #include "mf_internal.h"
 
 namespace mf {
@@ -37,54 +38,43 @@ struct __align__(16) LTile {
   int nt[8];               // tiles across the faces (-1: none)
 };
 
-// The tiles to visit are in a queue that all warps of the grid share: no barrier
-// between visits, and nobody waits for the longest visit of a sweep (with a grid
-// barrier per sweep over the active tiles, warps spent three quarters of their
-// time at it: one tile in a sweep of 500 used all its rounds, most a few).
+// The tiles to visit are in a queue that all warps of the grid share
+// (mf_tile_queue.cuh): no barrier between visits, and nobody waits for the longest
+// visit of a sweep (with a grid barrier per sweep over the active tiles, warps
+// spent three quarters of their time at it: one tile in a sweep of 500 used all
+// its rounds, most a few). Queues of successive phases alternate between two
+// buffers, and their counters between four sets; those of the phase before are
+// cleared while the next one runs.
 //
-// A tile is queued at most once. Its state word: QUEUED (it is in the queue, or,
-// while RUNNING, to be queued again after its visit), RUNNING (a warp has it),
-// and above them the faces whose inbox holds something (in a BFS: beyond which a
-// label fell) and, in a BFS, whether cells of the tile are seeds. A ticket (head)
-// names the queue place a warp waits for; an entry (tail) fills the next place.
-// Queues of successive phases alternate between two buffers, and their counters
-// between four sets; those of the phase before are cleared while the next one
-// runs.
-enum : int { QUEUED = 1, RUNNING = 2, FACES = 2, SEEDS = 64 << FACES };  // FACES: shift of the face bits
+// The queue's memory operations.
+struct QMem {
+  __device__ __forceinline__ int add(int *p, int x) { return atomicAdd(p, x); }
+  __device__ __forceinline__ int or_relaxed(int *p, int x) { return atomicOr(p, x); }
+  __device__ __forceinline__ int or_acquire(int *p, int x) {
+    int old;
+    asm volatile("atom.acquire.gpu.global.or.b32 %0, [%1], %2;" : "=r"(old) : "l"(p), "r"(x) : "memory");
+    return old;
+  }
+  __device__ __forceinline__ int and_acquire(int *p, int x) {
+    int old;
+    asm volatile("atom.acquire.gpu.global.and.b32 %0, [%1], %2;" : "=r"(old) : "l"(p), "r"(x) : "memory");
+    return old;
+  }
+  __device__ __forceinline__ int exch_acquire(int *p, int x) {
+    int old;
+    asm volatile("atom.acquire.gpu.global.exch.b32 %0, [%1], %2;" : "=r"(old) : "l"(p), "r"(x) : "memory");
+    return old;
+  }
+  __device__ __forceinline__ unsigned load(unsigned *p) { return *(volatile unsigned *)p; }
+  __device__ __forceinline__ void store(unsigned *p, unsigned x) { *(volatile unsigned *)p = x; }
+  __device__ __forceinline__ void release() { __threadfence(); }
+  __device__ __forceinline__ void acquire() { __threadfence(); }
+};
 
-// Places of a queue: at most `tiles` are filled, and at most one per warp of the
-// grid (2 tiles + 8, see lattice_grid) is waited for ahead of them.
-__host__ __device__ __forceinline__ int q_slots(const Lat &L) { return 3 * L.tiles + 8; }
-
-// Atomics on a tile's state whose result decides who queues it (acquire: what the
-// tile's last visit wrote is visible to whoever takes it from the queue then).
-__device__ __forceinline__ int state_or(int *p, int x) {
-  int old;
-  asm volatile("atom.acquire.gpu.global.or.b32 %0, [%1], %2;" : "=r"(old) : "l"(p), "r"(x) : "memory");
-  return old;
-}
-__device__ __forceinline__ int state_and(int *p, int x) {
-  int old;
-  asm volatile("atom.acquire.gpu.global.and.b32 %0, [%1], %2;" : "=r"(old) : "l"(p), "r"(x) : "memory");
-  return old;
-}
-
-// Place i of the queue: a sector of its own (idle warps look at neighbouring ones).
-constexpr int Q_STRIDE = 8;
-__device__ __forceinline__ int *q_place(const Dev &D, int ph, int i) {
-  return &D.lat.list[ph & 1][(size_t)(i % q_slots(D.lat)) * Q_STRIDE];
-}
-
-__device__ __forceinline__ void q_push(const Dev &D, int ph, int t) {
-  const int i = atomicAdd(&D.ctl->qtail[ph & 3], 1);
-  *(volatile int *)q_place(D, ph, i) = t + 1;
-}
-
-// Tile t has work (an inbox of a face in `faces`, or lower labels around it).
-// What the work consists of was written and fenced before.
-__device__ __forceinline__ void q_wake(const Dev &D, int ph, int t, int faces) {
-  const int old = state_or(&D.lat.state[t], QUEUED | (faces << FACES));
-  if (!(old & (QUEUED | RUNNING))) q_push(D, ph, t);
+// The queue of phase ph.
+__device__ __forceinline__ TileQueue<QMem> queue_of(const Dev &D, int ph) {
+  return TileQueue<QMem>{reinterpret_cast<unsigned *>(D.lat.list[ph & 1]), &D.ctl->qhead[ph & 3], &D.ctl->qtail[ph & 3],
+                         D.lat.state, D.lat.tiles, QMem{}};
 }
 
 // Between phases: empties the queue the phase before `ph` left (a push phase may
@@ -92,7 +82,8 @@ __device__ __forceinline__ void q_wake(const Dev &D, int ph, int t, int faces) {
 __device__ __forceinline__ void q_clear(const Dev &D, int ph) {
   const int tid = blockIdx.x * blockDim.x + threadIdx.x, nthr = gridDim.x * blockDim.x;
   if (tid == 0) D.ctl->qhead[(ph + 3) & 3] = D.ctl->qtail[(ph + 3) & 3] = D.ctl->qidle[(ph + 3) & 3] = 0;
-  for (int i = tid; i < q_slots(D.lat); i += nthr) *q_place(D, ph + 1, i) = 0;
+  const TileQueue<QMem> q = queue_of(D, ph + 1);
+  for (unsigned i = tid; i < q_slots(D.lat.tiles); i += nthr) *q.place(i) = 0;
 }
 
 // Takes the next tile (lane 0's work, the result in every lane); -1: the phase
@@ -105,20 +96,20 @@ __device__ __forceinline__ void q_clear(const Dev &D, int ph) {
 static __device__ int q_pop(const Dev &D, LShared &sh, int ph, bool timed, bool first) {
   int t = -1;
   if ((threadIdx.x & 31) == 0 && !(timed && !first && lat_timer() > sh.deadline)) {
-    const int ticket = atomicAdd(&D.ctl->qhead[ph & 3], 1);
-    int *slot = q_place(D, ph, ticket);
+    TileQueue<QMem> q = queue_of(D, ph);
+    const unsigned ticket = q.ticket();
     const bool looks = threadIdx.x == 0;
     const int nwarps = (int)gridDim.x * LW;
-    int v = *(volatile int *)slot;
-    if (!v) {
+    t = q.look(ticket);
+    if (t < 0) {
       atomicAdd(&D.ctl->qidle[ph & 3], 1);
       unsigned long long t0 = lat_timer();
       int tail0 = 0;
       // plain loads some way apart, few of them of the shared counters
       for (unsigned spins = 1;; spins++) {
         __nanosleep(spins < 8 ? 100 : 400);
-        v = *(volatile int *)slot;
-        if (v || *(volatile int *)&sh.done) break;
+        t = q.look(ticket);
+        if (t >= 0 || *(volatile int *)&sh.done) break;
         if (looks && (spins & 1)) {
           if (*(volatile int *)&D.ctl->qidle[ph & 3] == nwarps) {
             __threadfence();
@@ -144,34 +135,44 @@ static __device__ int q_pop(const Dev &D, LShared &sh, int ph, bool timed, bool 
           if (*(volatile int *)&D.ctl->err) break;
         }
       }
-      if (v) atomicAdd(&D.ctl->qidle[ph & 3], -1);
+      if (t >= 0) atomicAdd(&D.ctl->qidle[ph & 3], -1);
     }
-    __threadfence();  // what was written before the entry was made is visible from here on
-    if (v) {
-      *(volatile int *)slot = 0;
-      t = v - 1;
-    }
+    if (t >= 0) q.take(ticket);
   }
-  return __shfl_sync(LFULL, t, 0);
+  t = __shfl_sync(LFULL, t, 0);
+  __syncwarp();  // (a shuffle does not order memory) lane 0's fence holds for all lanes
+  return t;
 }
 
 // Starts the visit of tile t. Lane 0 gets the faces whose inbox holds something
 // (shifted by FACES), which the warp reads later with q_faces: the exchange is in
-// flight with the tile's loads. What the warps that woke t wrote before is
-// visible after it.
-__device__ __forceinline__ int q_begin(const Dev &D, int t) {
-  int old = 0;
-  if ((threadIdx.x & 31) == 0)
-    asm volatile("atom.acquire.gpu.global.exch.b32 %0, [%1], %2;" : "=r"(old) : "l"(&D.lat.state[t]), "r"((int)RUNNING) : "memory");
-  return old;
+// flight with the tile's loads.
+__device__ __forceinline__ int q_begin(const Dev &D, int ph, int t) {
+  return (threadIdx.x & 31) == 0 ? queue_of(D, ph).begin(t) : 0;
 }
-__device__ __forceinline__ int q_faces(int old) { return __shfl_sync(LFULL, old, 0) >> FACES; }
+__device__ __forceinline__ int q_faces(int old) {
+  old = __shfl_sync(LFULL, old, 0);
+  __syncwarp();  // what lane 0 acquired, every lane sees
+  return old >> FACES;
+}
 
-// Ends the visit of tile t after its results were fenced; `again`: it still has
-// work. Lane 0.
-__device__ __forceinline__ void q_end(const Dev &D, int ph, int t, bool again) {
-  if (again) atomicOr(&D.lat.state[t], (int)QUEUED);
-  if (state_and(&D.lat.state[t], ~RUNNING) & QUEUED) q_push(D, ph, t);
+// Ends the visit of tile t: the tiles across the faces in `out` have work now, and
+// t itself if `again`. All lanes; the warp's writes are released first.
+template <int DIM>
+__device__ __forceinline__ void q_done(const Dev &D, LTile<DIM> &w, int ph, int t, unsigned out, bool again) {
+  const int lane = threadIdx.x & 31;
+  TileQueue<QMem> q = queue_of(D, ph);
+  __syncwarp();  // also: the warp's tile may be overwritten
+  __threadfence();
+  int put = -1;
+  if (lane < Geo<DIM>::ND) {
+    if (((out >> lane) & 1) && q.mark(w.nt[lane], 1 << (lane ^ 1))) put = w.nt[lane];
+  } else if (lane == 31) {
+    if (q.end(t, again)) put = t;
+  }
+  __syncwarp();  // the pushes of all lanes together
+  if (put >= 0) q.push(put, lane < 31);
+  __syncwarp();  // the entries made are counted before lane 0 takes the next ticket
 }
 
 __device__ __forceinline__ void copy16(void *dst, const void *src) {
@@ -376,7 +377,7 @@ __device__ void push_visit(const Dev &D, LTile<DIM> &w, int t, int ph, int *drai
   using G = Geo<DIM>;
   const Lat &L = D.lat;
   const int lane = threadIdx.x & 31, cap = D.n_cap;
-  const int state = q_begin(D, t);
+  const int state = q_begin(D, ph, t);
 #pragma unroll 4
   for (int i = 0; i < G::ND * TV / 128; i++)
     copy16(&w.r[0][0] + 4 * (i * 32 + lane), &L.r[(size_t)t * G::ND * TV] + 4 * (i * 32 + lane));
@@ -439,12 +440,8 @@ __device__ void push_visit(const Dev &D, LTile<DIM> &w, int t, int ph, int *drai
     }
   }
   out = __reduce_or_sync(LFULL, out);
-  __threadfence();
-  __syncwarp();  // also: the warp's tile may be overwritten
-  if (lane < G::ND && ((out >> lane) & 1)) q_wake(D, ph, w.nt[lane], 1 << (lane ^ 1));
-  if (lane == 31) q_end(D, ph, t, n > 0);
+  q_done<DIM>(D, w, ph, t, out, n > 0);
   st.tiles_dis += lane == 0;
-  __syncwarp();  // the entries made are counted before lane 0 takes the next ticket
 }
 
 // One visit of a tile in a BFS phase by a warp: cells take better labels over the
@@ -460,7 +457,7 @@ __device__ void bfs_visit(const Dev &D, LTile<DIM> &w, int t, int ph, const unsi
   const int lane = threadIdx.x & 31;
   unsigned char *mk = reinterpret_cast<unsigned char *>(w.ex);
   copy16(mk + 16 * lane, mask + (size_t)t * TV + 16 * lane);
-  const int from = q_faces(q_begin(D, t)), faces = from & 63;
+  const int from = q_faces(q_begin(D, ph, t)), faces = from & 63;
   const bool seeds = from & (SEEDS >> FACES);
   load_labels<DIM>(D, w, t);
   asm volatile("cp.async.wait_all;" ::: "memory");
@@ -531,12 +528,8 @@ __device__ void bfs_visit(const Dev &D, LTile<DIM> &w, int t, int ph, const unsi
       need |= (unsigned)((__ldcg(&mask[(size_t)w.nt[j] * TV + G::cell(j ^ 1, f)]) >> (j ^ 1)) & 1) << j;
   }
   need = __reduce_or_sync(LFULL, need);
-  __threadfence();
-  __syncwarp();  // also: the warp's tile may be overwritten
-  if (lane < G::ND && ((need >> lane) & 1)) q_wake(D, ph, w.nt[lane], 1 << (lane ^ 1));
-  if (lane == 31) q_end(D, ph, t, false);
+  q_done<DIM>(D, w, ph, t, need, false);
   st.tiles_bfs += lane == 0;
-  __syncwarp();  // the entries made are counted before lane 0 takes the next ticket
 }
 
 // One CTA of 8 warps per SM, a tile (25 KB) per warp.
@@ -554,7 +547,7 @@ __global__ void __launch_bounds__(LT, 1) lattice3_kernel(Dev D) {
   __syncthreads();
   if (tid == 0) D.ctl->t_start = lat_timer();
   init_cells<DIM>(D);
-  for (int i = tid; i < q_slots(L); i += nthr) *q_place(D, 0, i) = *q_place(D, 1, i) = 0;
+  for (unsigned i = tid; i < q_slots(L.tiles); i += nthr) *queue_of(D, 0).place(i) = *queue_of(D, 1).place(i) = 0;
   bool ok = lat_sync(D, sh, 0);
   // Stages: phase 1 (excess toward t), phase 2 (what is left back to s), the cut.
   // A phase is a global relabel, visits until no tile is active or (gr_time_ratio)
@@ -571,7 +564,7 @@ __global__ void __launch_bounds__(LT, 1) lattice3_kernel(Dev D) {
     if (cutting) {
       const long long left = lat_sum(start_cut<DIM>(D, [&](int t) {
         L.state[t] = QUEUED | SEEDS;
-        q_push(D, ph, t);
+        queue_of(D, ph).push(t, false);
       }), sh.sum);
       if (threadIdx.x == 0 && left) {
         atomicAdd(reinterpret_cast<unsigned long long *>(&D.ctl->leftover), (unsigned long long)left);
@@ -583,7 +576,7 @@ __global__ void __launch_bounds__(LT, 1) lattice3_kernel(Dev D) {
           D, drain, [&](int t) { return __ldcg(&L.state[t]) >> FACES; },
           [&](int t, bool seeds) {
             L.state[t] = seeds ? QUEUED | SEEDS : 0;
-            if (seeds) q_push(D, ph, t);
+            if (seeds) queue_of(D, ph).push(t, false);
           });
     }
     ok = lat_sync(D, sh, 2);
@@ -596,7 +589,7 @@ __global__ void __launch_bounds__(LT, 1) lattice3_kernel(Dev D) {
     q_clear(D, ph);
     queue_active(D, [&](int t) {
       L.state[t] = QUEUED;
-      q_push(D, ph, t);
+      queue_of(D, ph).push(t, false);
     });
     ok = lat_sync(D, sh, 3);
     if (!ok) break;
@@ -637,9 +630,7 @@ __global__ void __launch_bounds__(LT, 1) lattice3_kernel(Dev D) {
 const void *lattice3_fn() { return (const void *)lattice3_kernel; }
 // Bytes of one tile queue.
 size_t lattice_queue_bytes(int tiles) {
-  Lat L;
-  L.tiles = tiles;
-  return (size_t)q_slots(L) * Q_STRIDE * 4;
+  return (size_t)q_slots(tiles) * Q_STRIDE * 4;
 }
 size_t lattice3_smem() { return LW * sizeof(LTile<3>); }
 
