@@ -48,6 +48,10 @@ struct __align__(16) LTile {
 //
 // The queue's memory operations.
 struct QMem {
+  const Dev *D;
+  unsigned long long deadline;  // end of a push phase (%globaltimer)
+  unsigned long long t0;
+
   __device__ __forceinline__ int add(int *p, int x) { return atomicAdd(p, x); }
   __device__ __forceinline__ int or_relaxed(int *p, int x) { return atomicOr(p, x); }
   __device__ __forceinline__ int or_acquire(int *p, int x) {
@@ -65,16 +69,31 @@ struct QMem {
     asm volatile("atom.acquire.gpu.global.exch.b32 %0, [%1], %2;" : "=r"(old) : "l"(p), "r"(x) : "memory");
     return old;
   }
+  __device__ __forceinline__ unsigned cas(unsigned *p, unsigned expect, unsigned x) { return atomicCAS(p, expect, x); }
   __device__ __forceinline__ unsigned load(unsigned *p) { return *(volatile unsigned *)p; }
   __device__ __forceinline__ void store(unsigned *p, unsigned x) { *(volatile unsigned *)p = x; }
   __device__ __forceinline__ void release() { __threadfence(); }
   __device__ __forceinline__ void acquire() { __threadfence(); }
+  // Wait for a place to become empty: given up when the phase ends (the warp whose
+  // entry lies there may have left at the deadline, and the relabel that follows
+  // queues afresh), after an error, and after D.timeout_ns.
+  __device__ __forceinline__ bool wait(unsigned spins) {
+    const unsigned long long now = lat_timer();
+    if (spins == 1) t0 = now;
+    if (now > deadline || *(volatile int *)&D->ctl->err) return false;
+    if (now - t0 > D->timeout_ns) {
+      lat_err(*D, MF_ERR_TIMEOUT, 4);
+      return false;
+    }
+    __nanosleep(100);
+    return true;
+  }
 };
 
-// The queue of phase ph.
-__device__ __forceinline__ TileQueue<QMem> queue_of(const Dev &D, int ph) {
+// The queue of phase ph, which ends by itself or at the deadline.
+__device__ __forceinline__ TileQueue<QMem> queue_of(const Dev &D, int ph, unsigned long long deadline = ~0ull) {
   return TileQueue<QMem>{reinterpret_cast<unsigned *>(D.lat.list[ph & 1]), &D.ctl->qhead[ph & 3], &D.ctl->qtail[ph & 3],
-                         D.lat.state, D.lat.tiles, QMem{}};
+                         D.lat.state, D.lat.tiles, QMem{&D, deadline, 0}};
 }
 
 // Between phases: empties the queue the phase before `ph` left (a push phase may
@@ -159,9 +178,10 @@ __device__ __forceinline__ int q_faces(int old) {
 // Ends the visit of tile t: the tiles across the faces in `out` have work now, and
 // t itself if `again`. All lanes; the warp's writes are released first.
 template <int DIM>
-__device__ __forceinline__ void q_done(const Dev &D, LTile<DIM> &w, int ph, int t, unsigned out, bool again) {
+__device__ __forceinline__ void q_done(const Dev &D, LTile<DIM> &w, int ph, unsigned long long deadline, int t, unsigned out,
+                                       bool again) {
   const int lane = threadIdx.x & 31;
-  TileQueue<QMem> q = queue_of(D, ph);
+  TileQueue<QMem> q = queue_of(D, ph, deadline);
   __syncwarp();  // also: the warp's tile may be overwritten
   __threadfence();
   int put = -1;
@@ -372,8 +392,8 @@ __device__ __forceinline__ int push_round(const Dev &D, LTile<DIM> &w, int t, in
 // a CTA per tile and two cells per thread, nearly every warp had one active lane
 // and a round took 1.3 us.
 template <int DIM>
-__device__ void push_visit(const Dev &D, LTile<DIM> &w, int t, int ph, int *drain, unsigned char *ret,
-                           LStat &st) {
+__device__ void push_visit(const Dev &D, LTile<DIM> &w, int t, int ph, unsigned long long deadline, int *drain,
+                           unsigned char *ret, LStat &st) {
   using G = Geo<DIM>;
   const Lat &L = D.lat;
   const int lane = threadIdx.x & 31, cap = D.n_cap;
@@ -440,7 +460,7 @@ __device__ void push_visit(const Dev &D, LTile<DIM> &w, int t, int ph, int *drai
     }
   }
   out = __reduce_or_sync(LFULL, out);
-  q_done<DIM>(D, w, ph, t, out, n > 0);
+  q_done<DIM>(D, w, ph, deadline, t, out, n > 0);
   st.tiles_dis += lane == 0;
 }
 
@@ -528,7 +548,7 @@ __device__ void bfs_visit(const Dev &D, LTile<DIM> &w, int t, int ph, const unsi
       need |= (unsigned)((__ldcg(&mask[(size_t)w.nt[j] * TV + G::cell(j ^ 1, f)]) >> (j ^ 1)) & 1) << j;
   }
   need = __reduce_or_sync(LFULL, need);
-  q_done<DIM>(D, w, ph, t, need, false);
+  q_done<DIM>(D, w, ph, ~0ull, t, need, false);
   st.tiles_bfs += lane == 0;
 }
 
@@ -612,7 +632,7 @@ __global__ void __launch_bounds__(LT, 1) lattice3_kernel(Dev D) {
     __syncthreads();
     unsigned char *const ret = stage == 2 ? L.ret : nullptr;
     bool first = true;
-    for (int t; (t = q_pop(D, sh, ph, true, first)) >= 0; first = false) push_visit<DIM>(D, w, t, ph, drain, ret, st);
+    for (int t; (t = q_pop(D, sh, ph, true, first)) >= 0; first = false) push_visit<DIM>(D, w, t, ph, sh.deadline, drain, ret, st);
     ok = lat_sync(D, sh, 4);
     if (timer) D.ctl->t_dis += lat_timer() - t1;
     if (ok && ph / 3 > D.max_rounds) {

@@ -7,6 +7,13 @@
 // label fell) and, in a BFS, whether cells of the tile are seeds. A ticket (head)
 // names the place a warp waits for; an entry (tail) fills the next place.
 //
+// Places are reused in turn, and an entry may still lie in its place when the
+// ring comes round to it, if the warp with its ticket has not looked since. So
+// an entry carries its lap, which only the ticket of that lap takes, and is
+// written only into an empty place. Fewer entries than places are out at a time
+// (a tile has one at most), so the ticket of an entry in the way has been drawn
+// and its warp is looking: the wait ends when it does.
+//
 // What a visit wrote is handed on twice: over the tile's state word, to whoever
 // queues it next, and over the entry, to the warp that takes it. Each hand-over
 // is a fence before the atomic that others read and a fence (or an acquire)
@@ -30,6 +37,7 @@ enum : int { QUEUED = 1, RUNNING = 2, FACES = 2, SEEDS = 64 << FACES };  // FACE
 MF_QUEUE_FN unsigned q_slots(int tiles) { return 3u * (unsigned)tiles + 8u; }
 
 constexpr int Q_STRIDE = 8;      // ints per place: a sector of its own (idle warps look at neighbouring ones)
+constexpr int Q_TILE_BITS = 23;  // of an entry: tile + 1 (there are at most 2^22 tiles); above them the lap
 
 template <class M>
 struct TileQueue {
@@ -40,14 +48,18 @@ struct TileQueue {
   M m;
 
   MF_QUEUE_FN unsigned *place(unsigned i) const { return ring + (size_t)(i % q_slots(tiles)) * Q_STRIDE; }
+  MF_QUEUE_FN unsigned entry(unsigned i, int t) const { return (i / q_slots(tiles)) << Q_TILE_BITS | (unsigned)(t + 1); }
 
   // Tile t joins the queue: `handed` after `mark` (what the last visitor of t wrote
   // was handed to this warp over the state word and is passed on), else after `end`
-  // (the visitor is this warp, whose writes the caller fenced).
-  MF_QUEUE_FN void push(int t, bool handed) {
+  // (the visitor is this warp, whose writes the caller fenced). False if the wait
+  // for the place was given up (M::wait).
+  MF_QUEUE_FN bool push(int t, bool handed) {
     const unsigned i = (unsigned)m.add(tail, 1);
     if (handed) m.release();
-    m.store(place(i), (unsigned)(t + 1));
+    for (unsigned spins = 1; m.cas(place(i), 0u, entry(i, t)) != 0; spins++)
+      if (!m.wait(spins)) return false;
+    return true;
   }
   // Tile t has work (an inbox of a face in `faces`, or lower labels around it):
   // true if it is to be pushed.
@@ -66,7 +78,8 @@ struct TileQueue {
   MF_QUEUE_FN unsigned ticket() { return (unsigned)m.add(head, 1); }
   // The tile in the place of ticket i, -1 if it is not there yet.
   MF_QUEUE_FN int look(unsigned i) {
-    return (int)m.load(place(i)) - 1;
+    const unsigned v = m.load(place(i));
+    return v && v >> Q_TILE_BITS == entry(i, 0) >> Q_TILE_BITS ? (int)(v & ((1u << Q_TILE_BITS) - 1)) - 1 : -1;
   }
   // The warp with ticket i has seen its tile and takes it.
   MF_QUEUE_FN void take(unsigned i) {

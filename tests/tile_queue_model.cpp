@@ -4,7 +4,8 @@
 //   race    a visit of a tile does not come after the last one, or not after the amounts it was woken for
 //   twice   two warps visit one tile at a time
 //   lost    work that nobody visits (the warps wait for ever)
-// argv: tiles warps visits seed mode hold (turns a warp is held up for, at most). Mode 0: the queue as it is; 1: entries are made without a release.
+// argv: tiles warps visits seed mode hold (turns a warp is held up for, at most). Mode 0: the queue as it is; 1: entries are made without a release; 2: entries
+// overwrite what lies in their place; 3: any ticket of a place takes its entry.
 #include <stddef.h>
 #include <stdio.h>
 #include <stdlib.h>
@@ -80,6 +81,13 @@ struct Mem {
   int or_acquire(int *p, int x) { return rmw(p, true, [x](int o) { return o | x; }); }
   int and_acquire(int *p, int x) { return rmw(p, true, [x](int o) { return o & x; }); }
   int exch_acquire(int *p, int x) { return rmw(p, true, [x](int) { return x; }); }
+  unsigned cas(unsigned *p, unsigned expect, unsigned x) {
+    if (mode == 2) {
+      store(p, x);
+      return 0;
+    }
+    return rmw(p, false, [expect, x](unsigned o) { return o == expect ? x : o; });
+  }
   unsigned load(unsigned *p) {
     turn();
     join(seen[cur], loc(p));
@@ -94,6 +102,10 @@ struct Mem {
     if (mode != 1) fence();
   }
   void acquire() { fence(); }
+  bool wait(unsigned spins) {
+    if (spins > 1000000) fail("lost");
+    return true;
+  }
 };
 
 int tiles, visits_left;
@@ -155,13 +167,18 @@ void warp() {
   mf::TileQueue<Mem> q = queue();
   for (;;) {
     const unsigned ticket = q.ticket();
-    int t = q.look(ticket);
+    auto look = [&]() {
+      if (mode != 3) return q.look(ticket);
+      const unsigned v = q.m.load(q.place(ticket));
+      return v ? (int)(v & ((1u << mf::Q_TILE_BITS) - 1)) - 1 : -1;
+    };
+    int t = look();
     if (t < 0) {
       idle++;
       for (unsigned spins = 0;; spins++) {
         if (rng() % 64 == 0) asleep[cur] = (int)(rng() % (unsigned)(hold + 1));  // a long sleep between two looks
         turn();
-        t = q.look(ticket);
+        t = look();
         if (t >= 0 || done) break;
         if (idle == nwarps && head == tail + nwarps) done = true;
         if (spins > 3000000) fail("lost");
@@ -200,7 +217,7 @@ int main(int argc, char **argv) {
   seen = out = now;
   for (int t = 0; t < tiles; t++) {  // queued before the phase (a grid barrier orders this before everything)
     state[t] = mf::QUEUED;
-    *queue().place((unsigned)t) = (unsigned)t + 1;
+    *queue().place((unsigned)t) = queue().entry((unsigned)t, t);
   }
   tail = tiles;
   std::vector<std::vector<char>> stack((size_t)nwarps, std::vector<char>(1 << 16));
