@@ -132,10 +132,11 @@ bool lattice_applies(const mf_graph *g) {
 }
 
 // Decides whether g (validated, on the device) is a lattice and sets g->lat
-// (dim 0: it is not). `scratch`: two ints of device memory.
+// (dim 0: it is not). Unions, of one instance too, run the list solver and are not
+// looked at. `scratch`: two ints of device memory.
 int lattice_detect(mf_graph *g, int *scratch, cudaStream_t st) {
   memset(&g->lat, 0, sizeof(g->lat));
-  if (g->ninst != 1 || g->max_degree > 8 || g->m == 0) return MF_OK;
+  if (g->vinst || g->max_degree > 8 || g->m == 0) return MF_OK;
   Lat L;
   memset(&L, 0, sizeof(L));
   L.s = g->s;

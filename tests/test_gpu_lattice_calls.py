@@ -74,3 +74,20 @@ def test_self_loops_have_their_flow_written(gpu, dims, where):
     assert np.array_equal(gpu.cut_bits_to_bool(cut.cpu().numpy().view(np.uint32), g.n), ref["cut"])
     assert f[at] == 0 and f[at + 1] == 0 and f.min() >= 0
     assert on_lists(stats)
+
+
+def test_unions_of_one_are_not_prepared_as_lattices(gpu):
+    """Batches and services run the list solver: a one-member union of a thin grid (whose padded tiles are several
+    times its cells) allocates no tiles."""
+    import torch
+
+    g = grid((60000, 5), 3)
+    csr = gpu.build_csr(g.n, g.tail, g.head, g.cap)
+    other = gpu.build_csr(g.n, np.append(g.tail, g.s), np.append(g.head, g.t), np.append(g.cap, 5).astype(np.int32))
+    used = []
+    for c in (csr, other):  # the second is no lattice
+        torch.cuda.synchronize()
+        before = torch.cuda.mem_get_info()[0]
+        with gpu.Batch([c], [(g.s, g.t)]):
+            used.append(before - torch.cuda.mem_get_info()[0])
+    assert abs(used[0] - used[1]) <= 8 << 20, used
