@@ -91,3 +91,19 @@ def test_unions_of_one_are_not_prepared_as_lattices(gpu):
         with gpu.Batch([c], [(g.s, g.t)]):
             used.append(before - torch.cuda.mem_get_info()[0])
     assert abs(used[0] - used[1]) <= 8 << 20, used
+
+
+@pytest.mark.parametrize("dims,lattice", [((2, 60000), True), ((2, 140000), False), ((40005, 8), True), ((40000, 7), False),
+                                          ((4, 5, 20000), True), ((3, 4, 40000), False), ((200, 3), True)])
+def test_thin_boxes_take_the_faster_solver(gpu, dims, lattice):
+    """More than 2,048 tiles that are mostly padding are left to the list solver."""
+    g = grid(dims, 5)
+    csr = gpu.build_csr(g.n, g.tail, g.head, g.cap)
+    ref = oracle.maxflow(g.n, g.s, g.t, g.tail, g.head, g.cap, want_flow=False)
+    with gpu.Graph.from_csr(csr, g.s, g.t) as G:
+        r = G.solve()
+        assert on_lattice(G.stats()) == lattice
+    cut = gpu.cut_bits_to_bool(r.cut_bits, g.n)
+    assert r.value == ref["value"] and np.array_equal(cut, ref["cut"])
+    f = np.where(csr.arc_slot >= 0, r.flow[np.maximum(csr.arc_slot, 0)], 0).astype(np.int64)
+    assert not oracle.check_flow(g.n, g.s, g.t, g.tail, g.head, g.cap, f, r.value, cut)
