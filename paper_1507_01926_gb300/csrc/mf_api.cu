@@ -263,7 +263,8 @@ int launch_config(mf_graph *g) {
   if (g->opt.blocks_per_sm > 0 && g->opt.blocks_per_sm < bps) bps = g->opt.blocks_per_sm;
   g->grid = bps * prop.multiProcessorCount;
   g->block = g->opt.block_threads;
-  return g->lat.dim ? lattice_grid(g, prop.multiProcessorCount, &g->lat_grid) : MF_OK;
+  lattice_options(g);
+  return lattice_applies(g) ? lattice_grid(g, prop.multiProcessorCount, &g->lat_grid) : MF_OK;
 }
 
 int check_options(const mf_options *o) {
@@ -649,18 +650,30 @@ static int solve_into(mf_graph *g, cudaStream_t st, int64_t *d_value, int32_t *d
   return run_kernel(g, D, st);
 }
 
+// Device memory of an output, kept with the graph. Tiles of a lattice in a buffer
+// of their own give way to it.
+static cudaError_t alloc_output(mf_graph *g, void **p, size_t bytes) {
+  cudaError_t e = cudaMalloc(p, bytes);
+  if (e == cudaErrorMemoryAllocation && lattice_give_up(g)) {
+    cudaGetLastError();
+    e = cudaMalloc(p, bytes);
+  }
+  if (e != cudaSuccess) *p = nullptr;
+  return e;
+}
+
 int mf_solve(mf_graph *g, int64_t *flow_value, int32_t *arc_flow, uint32_t *cut_bits) {
   clear_error();
   if (!g) return fail(MF_ERR_INVALID_ARG, "graph is NULL");
   cudaError_t e = cudaSetDevice(g->device);
   if (e != cudaSuccess) return cuda_fail(e, "cudaSetDevice");
   if (arc_flow && !g->d_flow) {
-    e = cudaMalloc((void **)&g->d_flow, (size_t)(g->m > 0 ? g->m : 1) * 4);
+    e = alloc_output(g, (void **)&g->d_flow, (size_t)(g->m > 0 ? g->m : 1) * 4);
     if (e != cudaSuccess) return cuda_fail(e, "cudaMalloc flow output");
   }
   const size_t words = ((size_t)g->n + 31) / 32;
   if (cut_bits && !g->d_cut) {
-    e = cudaMalloc((void **)&g->d_cut, words * 4);
+    e = alloc_output(g, (void **)&g->d_cut, words * 4);
     if (e != cudaSuccess) return cuda_fail(e, "cudaMalloc cut output");
   }
   int rc = solve_into(g, g->stream, nullptr, arc_flow ? g->d_flow : nullptr, cut_bits ? g->d_cut : nullptr);

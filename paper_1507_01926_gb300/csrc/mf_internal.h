@@ -18,7 +18,7 @@ struct mf_graph {
   mf_options opt{};
   mf_stats stats{};
   int grid = 0, block = 0;
-  mf::Lat lat{};               // lattice graphs: geometry and state (dim 0: not a lattice)
+  mf::Lat lat{};               // lattice graphs: geometry and state (dim 0: not a lattice; r null: state not placed)
   void *lat_buf = nullptr;     // the lattice state, where it does not fit the list solver's arrays
   int lat_grid = 0;            // CTAs of a lattice solve
   int ran_grid = 0;            // CTAs of the last solve
@@ -99,6 +99,8 @@ cudaError_t launch_solver(const Dev &D, int grid, int block, cudaStream_t stream
 int lattice_detect(mf_graph *g, int *scratch, cudaStream_t st);
 int lattice_grid(const mf_graph *g, int sms, int *grid);
 bool lattice_applies(const mf_graph *g);
+void lattice_options(mf_graph *g);
+bool lattice_give_up(mf_graph *g);
 cudaError_t launch_lattice(const Dev &D, int grid, cudaStream_t stream);
 int set_options(mf_graph *g, const mf_options *o);
 int autotune(mf_graph *g, const mf_tune_spec *spec, mf_options *best, double *best_ms);

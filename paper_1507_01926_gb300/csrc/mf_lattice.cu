@@ -84,10 +84,21 @@ __global__ void k_lat_check(int n, const int *row, const int *head, Lat L, int *
 
 }  // namespace
 
+// Options a lattice solve takes: the improved rounds with CTA-local lists, the
+// time-based relabel trigger (its only one) and the default CTA. Anything that
+// names a part of the list solver (simple rounds, gap relabeling, a round limit,
+// another CTA size, register budget or degree bin) runs there.
+bool lattice_applies(const mf_graph *g) {
+  const mf_options &o = g->opt;
+  return g->lat.dim && !o.simple_rounds && !o.gap_every && o.max_rounds == 0 && o.gr_time_ratio > 0 && o.block_threads == LT &&
+         o.kernel_variant == 0 && keep_local_limit(o, g->max_degree, o.block_threads) > 0;
+}
+
 // Places the tiled state in the list solver's arrays (both set their state up
 // from the capacities on every solve), or in a buffer of its own where the
 // padding of the last tiles makes it larger than those.
-static int lattice_place(mf_graph *g, Lat &L) {
+static int lattice_place(mf_graph *g) {
+  Lat &L = g->lat;
   const size_t cells = (size_t)L.tiles * TV, nd = 2 * (size_t)L.dim;
   const size_t faces = (size_t)L.tiles * nd * (L.dim == 3 ? 64 : 32);
   char *res = reinterpret_cast<char *>(g->rr), *vert = reinterpret_cast<char *>(g->vs);
@@ -121,18 +132,37 @@ static int lattice_place(mf_graph *g, Lat &L) {
   return MF_OK;
 }
 
-// Options a lattice solve takes: the improved rounds with CTA-local lists, the
-// time-based relabel trigger (its only one) and the default CTA. Anything that
-// names a part of the list solver (simple rounds, gap relabeling, a round limit,
-// another CTA size, register budget or degree bin) runs there.
-bool lattice_applies(const mf_graph *g) {
-  const mf_options &o = g->opt;
-  return g->lat.dim && !o.simple_rounds && !o.gap_every && o.max_rounds == 0 && o.gr_time_ratio > 0 && o.block_threads == LT &&
-         o.kernel_variant == 0 && keep_local_limit(o, g->max_degree, o.block_threads) > 0;
+// Gives the buffer of the tiled state back.
+static void lattice_unplace(mf_graph *g) {
+  gfree(g, g->lat_buf);
+  g->lat_buf = nullptr;
+  g->lat.r = nullptr;
 }
 
-// Decides whether g (validated, on the device) is a lattice and sets g->lat
-// (dim 0: it is not). Unions, of one instance too, run the list solver and are not
+// Called whenever g's options are set: the tiled state has its place while they
+// ask for lattice solves (a buffer of its own only then). Without memory for it
+// the list solver takes the graph from then on.
+void lattice_options(mf_graph *g) {
+  if (!g->lat.dim) return;
+  if (!lattice_applies(g)) {
+    if (g->lat_buf) lattice_unplace(g);
+  } else if (!g->lat.r && lattice_place(g) != MF_OK) {
+    clear_error();
+    g->lat.dim = 0;
+  }
+}
+
+// Where memory for a solve's outputs is short: gives the buffer of the tiled state
+// back and leaves g to the list solver. False if there is none.
+bool lattice_give_up(mf_graph *g) {
+  if (!g->lat_buf) return false;
+  lattice_unplace(g);
+  g->lat.dim = 0;
+  return true;
+}
+
+// Decides whether g (validated, on the device) is a lattice and sets the geometry in
+// g->lat (dim 0: it is not). Unions, of one instance too, run the list solver and are not
 // looked at. `scratch`: two ints of device memory.
 int lattice_detect(mf_graph *g, int *scratch, cudaStream_t st) {
   memset(&g->lat, 0, sizeof(g->lat));
@@ -177,11 +207,7 @@ int lattice_detect(mf_graph *g, int *scratch, cudaStream_t st) {
   }
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   if (e != cudaSuccess) return cuda_fail(e, "lattice check");
-  if (h[0]) return MF_OK;
-  if (lattice_place(g, L) == MF_OK)
-    g->lat = L;
-  else
-    clear_error();  // no memory for the padded tiles: the list solver takes the graph
+  if (!h[0]) g->lat = L;
   return MF_OK;
 }
 

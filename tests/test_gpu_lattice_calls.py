@@ -107,3 +107,42 @@ def test_thin_boxes_take_the_faster_solver(gpu, dims, lattice):
     assert r.value == ref["value"] and np.array_equal(cut, ref["cut"])
     f = np.where(csr.arc_slot >= 0, r.flow[np.maximum(csr.arc_slot, 0)], 0).astype(np.int64)
     assert not oracle.check_flow(g.n, g.s, g.t, g.tail, g.head, g.cap, f, r.value, cut)
+
+
+def test_tiles_take_memory_only_while_options_use_them(gpu):
+    """A thin grid's tiles are in a buffer of their own (here some 50 MB); a graph whose options keep it on the
+    list solver has none, and where the device has no room for an output they give way to it."""
+    import torch
+
+    g = grid((40000, 8), 6)
+    csr = gpu.build_csr(g.n, g.tail, g.head, g.cap)
+    lists = dict(max_rounds=2_000_000)  # the default limit, named: a list solve
+    torch.cuda.synchronize()
+
+    def free():
+        return torch.cuda.mem_get_info()[0]
+
+    before = free()
+    with gpu.Graph.from_csr(csr, g.s, g.t, gpu.default_options(**lists)) as G:
+        plain = before - free()
+        value = G.solve(flow=False, cut=False).value
+        assert on_lists(G.stats())
+        G.set_options(gpu.default_options())
+        tiled = before - free()
+        assert G.solve(flow=False, cut=False).value == value and on_lattice(G.stats())
+        assert tiled - plain >= 32 << 20
+        G.set_options(gpu.default_options(**lists))
+        assert before - free() <= plain + (4 << 20)
+        G.set_options(gpu.default_options())
+        torch.cuda.empty_cache()
+        rest = torch.empty(free() - (4 << 20), dtype=torch.uint8, device="cuda")  # leaves less than the flow needs
+        assert free() < 4 * G.m
+        try:
+            r = G.solve()
+        finally:
+            del rest
+            torch.cuda.empty_cache()
+        assert r.value == value and on_lists(G.stats())
+    f = np.where(csr.arc_slot >= 0, r.flow[np.maximum(csr.arc_slot, 0)], 0).astype(np.int64)
+    cut = gpu.cut_bits_to_bool(r.cut_bits, g.n)
+    assert not oracle.check_flow(g.n, g.s, g.t, g.tail, g.head, g.cap, f, r.value, cut)
