@@ -359,6 +359,9 @@ Dev make_dev(const mf_graph *g) {
   return D;
 }
 
+// CTAs of the kernel that a solve with D launches.
+static int solve_grid(const mf_graph *g, const Dev &D) { return D.lat.dim ? g->lat_grid : g->grid; }
+
 // The launch sequence of one solve: control-block reset, the persistent
 // kernel (between two timing events when `timed`), the read-back of the
 // control block.
@@ -366,9 +369,9 @@ static cudaError_t enqueue_solve(mf_graph *g, const Dev &D, cudaStream_t st, boo
   cudaError_t e;
   if ((e = cudaMemsetAsync(g->ctl, 0, sizeof(Ctl), st)) != cudaSuccess) return e;
   if (timed && (e = cudaEventRecord(g->ev0, st)) != cudaSuccess) return e;
-  e = D.lat.dim ? launch_lattice(D, g->lat_grid, st) : launch_solver(D, g->grid, g->block, st, g->opt.kernel_variant);
+  const int grid = solve_grid(g, D);
+  e = D.lat.dim ? launch_lattice(D, grid, st) : launch_solver(D, grid, g->block, st, g->opt.kernel_variant);
   if (e != cudaSuccess) return e;
-  g->ran_grid = D.lat.dim ? g->lat_grid : g->grid;
   if (timed && (e = cudaEventRecord(g->ev1, st)) != cudaSuccess) return e;
   return cudaMemcpyAsync(g->h_ctl, g->ctl, sizeof(Ctl), cudaMemcpyDeviceToHost, st);
 }
@@ -376,7 +379,7 @@ static cudaError_t enqueue_solve(mf_graph *g, const Dev &D, cudaStream_t st, boo
 // Captures the launch sequence for (D, st, launch shape) into g->gexec unless
 // the current capture already matches.
 static int ensure_graph(mf_graph *g, const Dev &D, cudaStream_t st) {
-  if (g->gexec && g->gstream == st && g->ggrid == g->grid && g->gblock == g->block &&
+  if (g->gexec && g->gstream == st && g->ggrid == solve_grid(g, D) && g->gblock == g->block &&
       g->gvariant == g->opt.kernel_variant && memcmp(&g->gdev, &D, sizeof(Dev)) == 0)
     return MF_OK;
   if (g->gexec) {
@@ -400,7 +403,7 @@ static int ensure_graph(mf_graph *g, const Dev &D, cudaStream_t st) {
   }
   g->gdev = D;
   g->gstream = st;
-  g->ggrid = g->grid;
+  g->ggrid = solve_grid(g, D);
   g->gblock = g->block;
   g->gvariant = g->opt.kernel_variant;
   return MF_OK;
@@ -435,6 +438,7 @@ int launch_kernel(mf_graph *g, Dev &D, cudaStream_t st) {
   } else {
     e = enqueue_solve(g, D, st, true);
   }
+  g->ran_grid = solve_grid(g, D);
   return e == cudaSuccess ? MF_OK : cuda_fail(e, "solver launch");
 }
 

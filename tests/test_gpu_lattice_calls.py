@@ -76,6 +76,24 @@ def test_self_loops_have_their_flow_written(gpu, dims, where):
     assert on_lists(stats)
 
 
+def test_capture_follows_the_launch_shape(gpu):
+    """A replayed solve takes a new blocks_per_sm, as a direct launch does."""
+    g = grid((700, 512), 2)  # 704 tiles
+    csr = gpu.build_csr(g.n, g.tail, g.head, g.cap)
+
+    def shapes(use_graph):
+        got = []
+        with gpu.Graph.from_csr(csr, g.s, g.t) as G:
+            for bps in (4, 3, 2, 4):
+                G.set_options(gpu.default_options(use_graph=use_graph, blocks_per_sm=bps))
+                value = G.solve(flow=False).value
+                assert on_lattice(G.stats())
+                got.append((value, G.stats()["grid_blocks"]))
+        return got
+
+    assert shapes(1) == shapes(0)
+
+
 def test_unions_of_one_are_not_prepared_as_lattices(gpu):
     """Batches and services run the list solver: a one-member union of a thin grid (whose padded tiles are several
     times its cells) allocates no tiles."""
