@@ -34,7 +34,9 @@
  * that only the list solver has: simple_rounds, gap_every and max_rounds 0,
  * gr_time_ratio > 0, block_threads 256, kernel_variant 0, local_lists on. Of the
  * options it then takes gr_time_ratio (its only relabel trigger), cut_only,
- * use_graph, timeout_ms and blocks_per_sm (2D). Same value and cut.
+ * use_graph, timeout_ms and blocks_per_sm (2D). Same value and cut. A lattice
+ * solve that does not end within 2,000,000 sweeps (2D) or visits of one warp (3D)
+ * is followed by a list solve, whose counters the statistics then are.
  *
  * Errors: every int-returning call returns MF_OK (0), MF_PENDING (1, only
  * mf_poll) or a negative MF_ERR_* code; mf_last_error() then describes the

@@ -20,6 +20,9 @@ BUILD = os.path.join(PKG, "_build")
 # the same library with every gather index of the solver checked (MF_CHECK_BOUNDS), for tests
 OUT_CHECK = os.path.join(PKG, "libmf_check.so")
 BUILD_CHECK = os.path.join(PKG, "_build_check")
+# the same library with lattice solves given up after a few sweeps or visits, for tests of what follows then
+OUT_LIMIT = os.path.join(PKG, "libmf_limit.so")
+BUILD_LIMIT = os.path.join(PKG, "_build_limit")
 
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 CU_SOURCES = ["mf_kernels_m0.cu", "mf_kernels_m1.cu", "mf_kernels_s0.cu", "mf_kernels_s1.cu", "mf_solver.cu", "mf_api.cu", "mf_batch.cu", "mf_service.cu", "mf_noalloc.cu", "mf_tune.cu", "mf_lattice.cu", "mf_lattice2.cu", "mf_lattice3.cu"]
@@ -91,6 +94,26 @@ def build(force: bool = False, verbose: bool = False, check: bool = False) -> st
     subprocess.check_call([nv, *ARCH, "-shared", "-o", tmp, *objs, "-lpthread"])
     os.replace(tmp, out)
     return out
+
+
+def build_limit() -> str:
+    """Builds libmf_limit.so: libmf.so but for the lattice kernels, compiled with a limit of 6 (MF_LATTICE_EFFORT)."""
+    build()
+    if up_to_date(OUT_LIMIT):
+        return OUT_LIMIT
+    os.makedirs(BUILD_LIMIT, exist_ok=True)
+    nv = nvcc()
+    kernels = ["mf_lattice2.cu", "mf_lattice3.cu"]
+    procs = [subprocess.Popen([nv, *ARCH, "-lineinfo", "-O3", "-std=c++17", "-I", INCLUDE, "-I", CSRC,
+                               "-DMF_LATTICE_EFFORT=6", "-Xcompiler", "-fPIC", "-c", os.path.join(CSRC, f), "-o",
+                               os.path.join(BUILD_LIMIT, f + ".o")]) for f in kernels]
+    if any([p.wait() for p in procs]):
+        raise RuntimeError("libmf_limit build failed")
+    objs = [os.path.join(BUILD_LIMIT if f in kernels else BUILD, f + ".o") for f in CU_SOURCES + CPP_SOURCES]
+    tmp = OUT_LIMIT + f".tmp{os.getpid()}"
+    subprocess.check_call([nv, *ARCH, "-shared", "-o", tmp, *objs, "-lpthread"])
+    os.replace(tmp, OUT_LIMIT)
+    return OUT_LIMIT
 
 
 if __name__ == "__main__":

@@ -409,13 +409,23 @@ static int ensure_graph(mf_graph *g, const Dev &D, cudaStream_t st) {
   return MF_OK;
 }
 
-// Runs the persistent kernel once with D; fills g->h_ctl and g->stats.
+// Runs the persistent kernel once with D; fills g->h_ctl and g->stats. A lattice
+// solve that was given up (its limit is not the user's max_rounds, with which the
+// list solver runs) is followed by a list solve; solve_ms is the time of both.
 int run_kernel(mf_graph *g, Dev &D, cudaStream_t st) {
-  const int rc = launch_kernel(g, D, st);
-  if (rc) return rc;
-  const cudaError_t e = cudaStreamSynchronize(st);
-  if (e != cudaSuccess) return cuda_fail(e, "solver");
-  return finish_kernel(g);
+  double given_up_ms = 0;
+  for (;;) {
+    int rc = launch_kernel(g, D, st);
+    if (rc) return rc;
+    const cudaError_t e = cudaStreamSynchronize(st);
+    if (e != cudaSuccess) return cuda_fail(e, "solver");
+    rc = finish_kernel(g);
+    g->stats.solve_ms += given_up_ms;
+    if (rc != MF_ERR_ITER_LIMIT || !D.lat.dim) return rc;
+    clear_error();
+    given_up_ms = g->stats.solve_ms;
+    memset(&D.lat, 0, sizeof(D.lat));
+  }
 }
 
 // Enqueues one solve with D on st (see run_kernel); returns without waiting.

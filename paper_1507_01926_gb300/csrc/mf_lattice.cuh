@@ -38,6 +38,12 @@
 //    order of pushes before that, the result is a maximum preflow (phase 1) or a
 //    flow (phase 2, the excess that is left back to s), so the value and S_min
 //    are exact.
+//  * That a solve ends is not proven: between two relabels labels only rise, but one
+//    that rose past its distance falls at the next relabel, and the list solver's
+//    argument (rounds whose labels stay below the distances) does not hold. So a
+//    solve is given up after LAT_EFFORT sweeps (2D) or visits of one warp (3D), far
+//    beyond any measured (256x256x128: 20,000 visits a warp), and the host runs the
+//    list solver on the graph.
 #include <cuda_runtime.h>
 #include <limits.h>
 
@@ -53,6 +59,10 @@ constexpr int LT = 256;      // threads per CTA
 constexpr int LW = LT / 32;
 constexpr int TV = 512;      // cells per tile: 32 x 16 or 8 x 8 x 8
 constexpr int LINF = UNV;    // label of a cell that does not reach the sink
+#ifndef MF_LATTICE_EFFORT      // (a test builds it with less)
+#define MF_LATTICE_EFFORT 2000000
+#endif
+constexpr int LAT_EFFORT = MF_LATTICE_EFFORT;
 
 template <int DIM>
 struct Geo {

@@ -111,10 +111,13 @@ __device__ __forceinline__ void q_clear(const Dev &D, int ph) {
 // does not change any more; the first warp of each CTA looks), or at the
 // deadline, which a warp's first tile of a phase does not heed (every phase gets
 // something done). A wait during which no tile is queued is bounded by
-// D.timeout_ns.
-static __device__ int q_pop(const Dev &D, LShared &sh, int ph, bool timed, bool first) {
+// D.timeout_ns, and a solve by LAT_EFFORT visits of this warp (a phase counts as
+// eight: its barriers and set-up), which also keeps the grid's tickets below 2^32.
+static __device__ int q_pop(const Dev &D, LShared &sh, int ph, bool timed, bool first, const LStat &st) {
   int t = -1;
-  if ((threadIdx.x & 31) == 0 && !(timed && !first && lat_timer() > sh.deadline)) {
+  const bool over = st.tiles_dis + st.tiles_bfs + 8u * (unsigned)ph > (unsigned)LAT_EFFORT;
+  if (over && (threadIdx.x & 31) == 0) lat_err(D, MF_ERR_ITER_LIMIT, 10);
+  if ((threadIdx.x & 31) == 0 && !over && !(timed && !first && lat_timer() > sh.deadline)) {
     TileQueue<QMem> q = queue_of(D, ph);
     const unsigned ticket = q.ticket();
     const bool looks = threadIdx.x == 0;
@@ -602,7 +605,7 @@ __global__ void __launch_bounds__(LT, 1) lattice3_kernel(Dev D) {
     ok = lat_sync(D, sh, 2);
     if (!ok) break;
     const unsigned char *const mask = cutting ? L.ret : L.mask;
-    for (int t; (t = q_pop(D, sh, ph, false, false)) >= 0;) bfs_visit<DIM>(D, w, t, ph, mask, st);
+    for (int t; (t = q_pop(D, sh, ph, false, false, st)) >= 0;) bfs_visit<DIM>(D, w, t, ph, mask, st);
     ok = lat_sync(D, sh, cutting ? 9 : 2);
     if (!ok || cutting) break;
     ph++;
@@ -632,13 +635,9 @@ __global__ void __launch_bounds__(LT, 1) lattice3_kernel(Dev D) {
     __syncthreads();
     unsigned char *const ret = stage == 2 ? L.ret : nullptr;
     bool first = true;
-    for (int t; (t = q_pop(D, sh, ph, true, first)) >= 0; first = false) push_visit<DIM>(D, w, t, ph, sh.deadline, drain, ret, st);
+    for (int t; (t = q_pop(D, sh, ph, true, first, st)) >= 0; first = false) push_visit<DIM>(D, w, t, ph, sh.deadline, drain, ret, st);
     ok = lat_sync(D, sh, 4);
     if (timer) D.ctl->t_dis += lat_timer() - t1;
-    if (ok && ph / 3 > D.max_rounds) {
-      lat_err(D, MF_ERR_ITER_LIMIT, 10);
-      ok = false;
-    }
   }
   if (ok) write_outputs<DIM>(D);
   add_stats(D, sh, st);

@@ -164,3 +164,27 @@ def test_tiles_take_memory_only_while_options_use_them(gpu):
     f = np.where(csr.arc_slot >= 0, r.flow[np.maximum(csr.arc_slot, 0)], 0).astype(np.int64)
     cut = gpu.cut_bits_to_bool(r.cut_bits, g.n)
     assert not oracle.check_flow(g.n, g.s, g.t, g.tail, g.head, g.cap, f, r.value, cut)
+
+
+@pytest.mark.parametrize("opts", [{}, dict(cut_only=1), dict(use_graph=1)])
+@pytest.mark.parametrize("dims", [(150, 130), (20, 30, 25)])
+def test_solves_that_are_given_up_end_on_the_list_solver(gpu, dims, opts):
+    """With the lattice kernels built to give up after a few sweeps or visits, every solve still has its result."""
+    from paper_1507_01926_gb300 import build as mfbuild
+
+    g = grid(dims, 8)
+    csr = gpu.build_csr(g.n, g.tail, g.head, g.cap)
+    ref = oracle.maxflow(g.n, g.s, g.t, g.tail, g.head, g.cap, want_flow=False)
+    before = gpu.use_library(mfbuild.build_limit())
+    try:
+        with gpu.Graph.from_csr(csr, g.s, g.t, gpu.default_options(**opts)) as G:
+            for _ in range(2):
+                r = G.solve(flow=not opts.get("cut_only"))
+                assert on_lists(G.stats())
+                cut = gpu.cut_bits_to_bool(r.cut_bits, g.n)
+                assert r.value == ref["value"] and np.array_equal(cut, ref["cut"])
+                if r.flow is not None:
+                    f = np.where(csr.arc_slot >= 0, r.flow[np.maximum(csr.arc_slot, 0)], 0).astype(np.int64)
+                    assert not oracle.check_flow(g.n, g.s, g.t, g.tail, g.head, g.cap, f, r.value, cut)
+    finally:
+        gpu.use_library(before)
