@@ -178,9 +178,13 @@ typedef struct mf_options {
 /* Counters of the last solve. Arc scans count every slot examined by a
  * discharge pass (a relabel pass of the simple rounds) or a BFS expansion,
  * slots with zero residual included; scans_discharge_residual counts the
- * discharge scans of slots with positive residual. Of a lattice solve, rounds and
- * bfs_levels count sweeps over the tiles (2D) or visits of tiles (3D), the other
- * counters cells and their slots; the CTA 0 times and rounds_by_size stay 0. */
+ * discharge scans of slots with positive residual. Lattice solves: rounds and
+ * bfs_levels count sweeps over the tiles (2D) or visits of tiles (3D), and the CTA 0
+ * times and rounds_by_size stay 0. Volumes count slots: those of a discharged cell to
+ * its neighbours and to the phase's sink, and in BFS those to the neighbours of every
+ * cell that offers its label. Images count directions, whether or not the cell has a
+ * slot there: 5 per discharge of a cell, and in BFS the 4 of every cell of a visited
+ * tile, once per visit; scans_discharge_residual stays 0. */
 typedef struct mf_stats {
   int64_t rounds;           /* push-relabel rounds, both phases */
   int64_t rounds_phase1;

@@ -103,6 +103,7 @@ struct Lat {
   int *inbox;          // per tile, face and face entry: amounts pushed over that face, not taken in yet
   unsigned char *mask; // per cell, bit j: residual in direction j (set by a global relabel)
   unsigned char *ret;  // per cell: excess was returned to s; then the mask of the cut
+  unsigned char *slots;  // 3D, per cell, for the counts of scans: its slots to neighbours, + 8: one to t, + 16: one to s
   int *list[2];        // 2D: tile lists by generation parity; 3D: tile queues by phase parity
   int *state;          // per tile. 2D: last sweep it was queued for; 3D: queued, running, faces with an inbox
   int *bits;           // 2D: 2 x tiles, by sweep parity: faces whose inbox holds something

@@ -104,7 +104,7 @@ static int lattice_place(mf_graph *g) {
   char *res = reinterpret_cast<char *>(g->rr), *vert = reinterpret_cast<char *>(g->vs);
   char *bfs = reinterpret_cast<char *>(g->blab);
   int *list[3] = {g->list[0], g->list[1], g->list[2]};
-  const size_t nres = cells * nd * 4, nvert = cells * 20, nbfs = faces * 4 + cells * 2;
+  const size_t nres = cells * nd * 4, nvert = cells * (L.dim == 3 ? 21 : 20), nbfs = faces * 4 + cells * 2;
   const size_t queue = lattice_queue_bytes(L.tiles);
   if (nres > (size_t)g->m * 8 || nvert > (size_t)g->n * sizeof(VRec) || nbfs > (size_t)g->n * 8 ||
       2 * queue > (size_t)g->n * 4) {
@@ -122,6 +122,7 @@ static int lattice_place(mf_graph *g) {
   L.d = reinterpret_cast<int *>(L.ex + cells);
   L.drain = L.d + cells;
   L.back = L.drain + cells;
+  L.slots = reinterpret_cast<unsigned char *>(L.back + cells);
   L.inbox = reinterpret_cast<int *>(bfs);
   L.mask = reinterpret_cast<unsigned char *>(L.inbox + faces);
   L.ret = L.mask + cells;

@@ -180,6 +180,12 @@ __device__ __forceinline__ int next_tile(const Lat &L, int t, int j) {
   return (j & 1) ? (at + 1 < end ? t + st : -1) : (at > 0 ? t - st : -1);
 }
 
+// Scans count what a lattice solve looks at. Volumes: slots of the graph (Lat::slots),
+// of a discharged cell those to its neighbours and the one to the phase's sink, in
+// a BFS those to the neighbours of a cell that offers its label. Images: directions,
+// with a slot or without, the drain among them once per visit of a cell; in a BFS
+// those of all cells of a visited tile once per visit (counting slots cost 2-4% of a
+// solve there: 64 registers, and a round's work is little more than the count).
 struct LStat {
   unsigned tiles_dis = 0, tiles_bfs = 0;  // visits of tiles
   unsigned scans_dis = 0, scans_res = 0, scans_bfs = 0, pushes = 0, relabels = 0, visits_dis = 0, visits_bfs = 0;
@@ -357,7 +363,7 @@ __device__ __forceinline__ void init_cells(const Dev &D) {
     for (int c = 0; c < 2; c++) {
       const int u = threadIdx.x + c * LT, p = cell_at<DIM>(L, t, u);
       long long ex = 0;
-      int dr = 0, rs = 0, r[G::ND];
+      int dr = 0, rs = 0, slots = 0, r[G::ND];
 #pragma unroll
       for (int j = 0; j < G::ND; j++) r[j] = 0;
       if (p >= 0) {
@@ -367,12 +373,15 @@ __device__ __forceinline__ void init_cells(const Dev &D) {
           const int w = __ldg(&D.head[a]), cp = __ldg(&D.cap[a]);
           if (w == L.t) {
             dr = cp;
+            slots += 8;
           } else if (w == L.s) {
+            slots += 16;
             const int cs = __ldg(&D.cap[__ldg(&D.rev[a])]);
             rs = cp + cs;
             ex = cs;
           } else {
             const int jj = dir_of<DIM>(L, p, cell_of(L, w));
+            slots++;
 #pragma unroll
             for (int j = 0; j < G::ND; j++)
               if (j == jj) r[j] = cp;
@@ -384,6 +393,7 @@ __device__ __forceinline__ void init_cells(const Dev &D) {
       L.drain[at] = dr;
       L.back[at] = rs;
       L.ret[at] = 0;
+      if (DIM == 3) L.slots[at] = (unsigned char)slots;
 #pragma unroll
       for (int j = 0; j < G::ND; j++) L.r[((size_t)t * G::ND + j) * TV + u] = r[j];
     }

@@ -34,6 +34,7 @@ struct __align__(16) LTile {
     unsigned short q[TV];    // the cells of this round
     int got[Geo<DIM>::NH];   // while loading: amounts from the inbox, by face entry
   };
+  __align__(16) unsigned char slots[TV];  // Lat::slots
   unsigned inq[TV / 32];   // bitmap of the cells of the next round
   int nt[8];               // tiles across the faces (-1: none)
 };
@@ -335,7 +336,8 @@ __device__ __forceinline__ int push_round(const Dev &D, LTile<DIM> &w, int t, in
       e -= left;
       dr = w.drain[u];
       st.visits_dis++;
-      st.scans_dis += G::ND + 1;
+      st.scans_dis += (w.slots[u] & 7) + ((w.slots[u] >> (ret ? 4 : 3)) & 1);
+      st.scans_res += dr > 0;
       if (dr > 0 && left > 0) {  // the drain is an arc to label 0
         const int a = min(dr, left);
         w.drain[u] = dr -= a;
@@ -408,6 +410,7 @@ __device__ void push_visit(const Dev &D, LTile<DIM> &w, int t, int ph, unsigned 
   for (int i = 0; i < TV / 64; i++) copy16(&w.ex[2 * (i * 32 + lane)], &L.ex[(size_t)t * TV + 2 * (i * 32 + lane)]);
 #pragma unroll
   for (int i = 0; i < TV / 128; i++) copy16(&w.drain[4 * (i * 32 + lane)], &drain[(size_t)t * TV + 4 * (i * 32 + lane)]);
+  copy16(w.slots + 16 * lane, &L.slots[(size_t)t * TV + 16 * lane]);
   load_labels<DIM>(D, w, t);  // (a halo older than the inbox is as good)
   const int bits = q_faces(state);
   if (bits) {
@@ -480,6 +483,7 @@ __device__ void bfs_visit(const Dev &D, LTile<DIM> &w, int t, int ph, const unsi
   const int lane = threadIdx.x & 31;
   unsigned char *mk = reinterpret_cast<unsigned char *>(w.ex);
   copy16(mk + 16 * lane, mask + (size_t)t * TV + 16 * lane);
+  copy16(w.slots + 16 * lane, &L.slots[(size_t)t * TV + 16 * lane]);
   const int from = q_faces(q_begin(D, ph, t)), faces = from & 63;
   const bool seeds = from & (SEEDS >> FACES);
   load_labels<DIM>(D, w, t);
@@ -500,7 +504,6 @@ __device__ void bfs_visit(const Dev &D, LTile<DIM> &w, int t, int ph, const unsi
       }
     }
     __syncwarp();
-    st.scans_bfs += G::FS / 32;
   }
   n = next_list<DIM>(w, touched);
   if (seeds) {  // first visit: every cell with a label offers it
@@ -530,7 +533,7 @@ __device__ void bfs_visit(const Dev &D, LTile<DIM> &w, int t, int ph, const unsi
             atomicMin(&w.lab[q + G::pstep(j)], l);
             mark<DIM>(w, u + G::step(j));
           }
-        st.scans_bfs += G::ND;
+        st.scans_bfs += w.slots[u] & 7;
         st.visits_bfs++;
       }
     n = next_list<DIM>(w, touched);

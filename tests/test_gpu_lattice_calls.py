@@ -188,3 +188,24 @@ def test_solves_that_are_given_up_end_on_the_list_solver(gpu, dims, opts):
                     assert not oracle.check_flow(g.n, g.s, g.t, g.tail, g.head, g.cap, f, r.value, cut)
     finally:
         gpu.use_library(before)
+
+
+@pytest.mark.parametrize("cut_only", [0, 1])
+def test_volume_scans_count_slots_that_exist(gpu, cut_only):
+    """Arcs along the slowest axis only (and one along each other, which make the box known): a cell has at most two
+    slots to neighbours and one to a terminal; four cells have one more."""
+    dims = (20, 24, 22)
+    g = grid(dims, 9)
+    cell = (g.tail < g.s) & (g.head < g.s)
+    step = np.where(cell, np.abs(g.tail - g.head), 0)
+    keep = ~cell | (step == 24 * 22)
+    for k in (1, 22):
+        keep[np.flatnonzero(step == k)[0]] = True
+    csr = gpu.build_csr(g.n, g.tail[keep], g.head[keep], g.cap[keep])
+    with gpu.Graph.from_csr(csr, g.s, g.t, gpu.default_options(cut_only=cut_only)) as G:
+        G.solve(flow=False)
+        st = G.stats()
+    assert on_lattice(st) and st["visits_discharge"] > 0 and st["visits_bfs"] > 0
+    assert st["scans_discharge"] <= 3 * st["visits_discharge"] + 4 * 16 * st["rounds"]  # 16 rounds a visit at most
+    assert 0 < st["scans_discharge_residual"] <= st["scans_discharge"]
+    assert st["scans_bfs"] <= 2.1 * st["visits_bfs"]
