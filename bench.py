@@ -47,6 +47,12 @@ B_VISIT_BFS = 16    # BFS frontier vertex: row offsets 8 + list 8
 B_SLOT_FIXED = 20   # per solve and slot: residual reset (cap 4 + write 4) + flow output (cap 4 + res 4 + out 4)
 B_VERTEX_FIXED = 28  # per solve and vertex: state reset (d 4 + e 8 + addedExcess 8 + stamps 4) + cut 4
 B_VERTEX_GR = 12    # per global relabel and vertex: label reset 4 + rebuild (label 4 + excess ... 4)
+# What the lattice solver for volumes moves between the SMs and L2 / HBM, per unit (a tile has 512 cells):
+B_TILE_PUSH = 22528  # push visit, loads: residuals 24, excess 8, sink residual 4, label 4, slot count 1 per cell; halo 1536
+B_TILE_BFS = 4608    # BFS visit, loads: label 4, mask 1, slot count 1 per cell; halo 1536
+B_CELL_GR = 45       # per global relabel and cell: residuals 24, sink residual 4, mask 1, label 4; active check 12
+B_CELL_INIT = 45     # per solve and cell: state 42 and inbox 3 written
+B_SLOT_LATTICE = 24  # per solve and slot: head 4 + cap 4 read; flow output: head, cap, residual read, flow written
 HBM_NOMINAL_GBS = 7900.0  # GB300 HBM3e, nominal (the measured copy peak is the roofline's denominator)
 
 
@@ -67,6 +73,36 @@ def phase_rooflines(st: dict, n: int, peak: float) -> dict:
         gbs = b / (ms * 1e6) if ms > 0 else None
         out[name] = {"model_bytes": int(b), "ms": ms, "achieved_GBps": gbs, "frac": gbs / peak if gbs else None}
     return out
+
+
+def lattice_model_bytes(st: dict, dims, n: int, m: int) -> int:
+    """Bytes the tile visits and the passes over all cells of a volume's lattice solve load, and its fixed reads and
+    writes (the stores of a visit, of the cells that took part, are not counted). L2 and HBM traffic together."""
+    cells = 512
+    for d in dims:
+        cells *= (d + 7) // 8
+    return int(B_TILE_PUSH * st["rounds"] + B_TILE_BFS * st["bfs_levels"] + B_CELL_GR * cells * st["global_relabels"]
+               + B_CELL_INIT * cells + B_SLOT_LATTICE * m + 8 * n)
+
+
+def grid_roofline(stats: list, n: int, m: int, dims, ms: float, peak: float, peak_kind: str, traffic_of) -> dict:
+    """The roofline entry of the 3D-grid line: one launch of the solve's only kernel takes `ms` on average; stats of the
+    timed solves; traffic_of(kernel): DRAM bytes per launch from a stored profile of that kernel version, or None.
+    A lattice solve counts no rounds by size. Its work is rounds in shared memory: the list solver's bytes per scan
+    and visit say nothing about it, and its phases are not split."""
+    lattice = not any(stats[-1]["rounds_by_size"])
+    kernel = "mf::lattice3_kernel" if lattice else "mf::solve_kernel"
+    per = [lattice_model_bytes(s, dims, n, m) if lattice else model_bytes(s, n, m) for s in stats]
+    achieved = statistics.mean(per) / (ms / 1000.0) / 1e9
+    traffic = traffic_of(kernel)
+    return {"bound": "latency" if lattice else "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
+            "frac": achieved / peak, "traffic": traffic, "peak_kind": peak_kind, "kernel": kernel,
+            "model": "bytes loaded by tile visits and passes over the cells, L2 and HBM together" if lattice
+                     else "algorithmic bytes of the list solver's scans, visits and pushes",
+            "peak_nominal": HBM_NOMINAL_GBS, "frac_nominal": achieved / HBM_NOMINAL_GBS,
+            "traffic_GBps": (traffic / (ms / 1000.0) / 1e9) if traffic else None,
+            "model_bytes_per_launch": statistics.mean(per),
+            "phases": None if lattice else phase_rooflines(stats[len(stats) // 2], n, peak)}
 
 
 def paired_slot_count(tail, head) -> int:
@@ -180,13 +216,26 @@ def load_workload(shape=None):
     return g, csr
 
 
-def kernel_source_hash() -> str:
-    """Identifies the solver kernel version the stored ncu counters belong to."""
+KERNEL_SOURCES = {"mf::solve_kernel": ("mf_solver.cuh", "mf_device.cuh"),
+                  "mf::lattice3_kernel": ("mf_lattice3.cu", "mf_lattice.cuh", "mf_tile_queue.cuh", "mf_device.cuh")}
+
+
+def kernel_source_hash(kernel: str = "mf::solve_kernel") -> str:
+    """Identifies the kernel version the stored ncu counters belong to."""
     import hashlib
 
     csrc = os.path.join(ROOT, "paper_1507_01926_gb300", "csrc")
-    data = b"".join(open(os.path.join(csrc, f), "rb").read() for f in ("mf_solver.cuh", "mf_device.cuh"))
+    data = b"".join(open(os.path.join(csrc, f), "rb").read() for f in KERNEL_SOURCES[kernel])
     return hashlib.sha256(data).hexdigest()[:16]
+
+
+def stored_traffic(kernel: str):
+    """DRAM bytes per launch of the 256x256x128 grid from the stored profile of this very kernel version, or None."""
+    p = os.path.join(ROOT, "profiles", kernel.split("::")[1] + "_grid3d_256x256x128.json")
+    if not os.path.exists(p):
+        return None
+    rec = json.load(open(p))
+    return rec.get("dram_bytes_per_launch") if rec.get("kernel_source_sha256_16") == kernel_source_hash(kernel) else None
 
 
 def golden_record():
@@ -648,18 +697,10 @@ def main():
     grec = golden_record() if tuple(args.grid3d) == (256, 256, 128) else None
     gold = grec["value"] if grec else None
 
-    # roofline of the (only) kernel: the persistent solve kernel, one launch per step. The lattice solver, which
-    # counts no rounds by size, does most of the model's accesses in shared memory: its figure is not HBM traffic
-    kernel = "mf::solve_kernel" if any(stats[-1]["rounds_by_size"]) else "mf::lattice3_kernel"
     peak, peak_kind = peaks()
-    mb = [model_bytes(s, g.n, csr.m) for s in stats]
-    achieved = (sum(mb) / len(mb)) / (statistics.mean(per_step) / 1000.0) / 1e9
-    traffic = None
-    tp = os.path.join(ROOT, "profiles", "solve_kernel_grid3d_256x256x128.json")
-    if os.path.exists(tp) and tuple(args.grid3d) == (256, 256, 128):
-        rec = json.load(open(tp))
-        if rec.get("kernel_source_sha256_16") == kernel_source_hash():
-            traffic = rec.get("dram_bytes_per_launch")  # counters of this very kernel version
+    full_size = tuple(args.grid3d) == (256, 256, 128)
+    roofline = grid_roofline(stats, g.n, csr.m, args.grid3d, statistics.mean(per_step), peak, peak_kind,
+                             stored_traffic if full_size else lambda kernel: None)
 
     if rank != 0:
         G.close()
@@ -719,12 +760,7 @@ def main():
                                  if grec else None),
         "rounds": stats[-1]["rounds"], "global_relabels": stats[-1]["global_relabels"],
         "scans_per_solve": scans / args.steps,
-        "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
-                     "traffic": traffic, "peak_kind": peak_kind, "kernel": kernel,
-                     "peak_nominal": HBM_NOMINAL_GBS, "frac_nominal": achieved / HBM_NOMINAL_GBS,
-                     "traffic_GBps": (traffic / (statistics.mean(per_step) / 1000.0) / 1e9) if traffic else None,
-                     "model_bytes_per_launch": statistics.mean(mb),
-                     "phases": phase_rooflines(stats[len(stats) // 2], g.n, peak)},
+        "roofline": roofline,
         "cpu_baseline": cpu, "e2e": e2e, "clocks": clocks, "gpu_launches": args.steps,
         "grid": [warm_stats["grid_blocks"], warm_stats["block_threads"]],
         "options": {"tuned": ("cached autotuner choice" if hit else "defaults (no cached choice)")
