@@ -346,8 +346,9 @@ void mf_batch_destroy(mf_batch *b);
  * (128, 4), (256, 1)}, kernel_variant {0..4} (and variant 4 with
  * bin_thread 16), local_lists {0, 1}, bfs_hops {1, 4, 8, 16} (these two
  * only on graphs where they act) and bfs_pull {0, 20, 50, 200},
- * starting from g's current options; candidates that are invalid together or
- * do not fit the GPU are skipped. A candidate's time is the median device time of spec->reps solves
+ * starting from g's current options; candidates that are invalid together, that
+ * do not fit the GPU, or that differ from the best so far only in options their
+ * lattice solve does not read (see Lattices above) are skipped. A candidate's time is the median device time of spec->reps solves
  * (maximum flow value only, no per-arc outputs); spec->sweeps passes over the
  * coordinates at most (fewer when a pass changes nothing); no new candidate
  * starts once the solves took spec->time_budget_ms (0 = no limit). spec may

@@ -264,7 +264,7 @@ int launch_config(mf_graph *g) {
   g->grid = bps * prop.multiProcessorCount;
   g->block = g->opt.block_threads;
   lattice_options(g);
-  return lattice_applies(g) ? lattice_grid(g, prop.multiProcessorCount, &g->lat_grid) : MF_OK;
+  return lattice_applies(g, g->opt) ? lattice_grid(g, prop.multiProcessorCount, &g->lat_grid) : MF_OK;
 }
 
 int check_options(const mf_options *o) {
@@ -657,7 +657,7 @@ void mf_destroy_graph(mf_graph *g) {
 static int solve_into(mf_graph *g, cudaStream_t st, int64_t *d_value, int32_t *d_flow, uint32_t *d_cut) {
   if (g->opt.cut_only && d_flow) return fail(MF_ERR_INVALID_ARG, "cut_only solves produce no per-arc flow");
   Dev D = make_dev(g);
-  if (lattice_applies(g)) D.lat = g->lat;
+  if (lattice_applies(g, g->opt)) D.lat = g->lat;
   D.out_value = d_value ? reinterpret_cast<long long *>(d_value) : g->d_value;
   D.out_flow = d_flow;
   D.out_cut = d_cut;

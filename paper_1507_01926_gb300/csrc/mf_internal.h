@@ -98,7 +98,7 @@ int solver_occupancy(int block_threads, int *blocks_per_sm, int variant, bool mu
 cudaError_t launch_solver(const Dev &D, int grid, int block, cudaStream_t stream, int variant);
 int lattice_detect(mf_graph *g, int *scratch, cudaStream_t st);
 int lattice_grid(const mf_graph *g, int sms, int *grid);
-bool lattice_applies(const mf_graph *g);
+bool lattice_applies(const mf_graph *g, const mf_options &o);
 void lattice_options(mf_graph *g);
 bool lattice_give_up(mf_graph *g);
 cudaError_t launch_lattice(const Dev &D, int grid, cudaStream_t stream);

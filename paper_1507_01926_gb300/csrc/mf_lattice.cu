@@ -88,8 +88,7 @@ __global__ void k_lat_check(int n, const int *row, const int *head, Lat L, int *
 // time-based relabel trigger (its only one) and the default CTA. Anything that
 // names a part of the list solver (simple rounds, gap relabeling, a round limit,
 // another CTA size, register budget or degree bin) runs there.
-bool lattice_applies(const mf_graph *g) {
-  const mf_options &o = g->opt;
+bool lattice_applies(const mf_graph *g, const mf_options &o) {
   return g->lat.dim && !o.simple_rounds && !o.gap_every && o.max_rounds == 0 && o.gr_time_ratio > 0 && o.block_threads == LT &&
          o.kernel_variant == 0 && keep_local_limit(o, g->max_degree, o.block_threads) > 0;
 }
@@ -145,7 +144,7 @@ static void lattice_unplace(mf_graph *g) {
 // the list solver takes the graph from then on.
 void lattice_options(mf_graph *g) {
   if (!g->lat.dim) return;
-  if (!lattice_applies(g)) {
+  if (!lattice_applies(g, g->opt)) {
     if (g->lat_buf) lattice_unplace(g);
   } else if (!g->lat.r && lattice_place(g) != MF_OK) {
     clear_error();

@@ -25,7 +25,7 @@ namespace {
 // *ms = device time of the kernel.
 int timed_solve(mf_graph *g, double *ms, std::vector<long long> *values) {
   Dev D = make_dev(g);
-  if (lattice_applies(g)) D.lat = g->lat;
+  if (lattice_applies(g, g->opt)) D.lat = g->lat;
   D.out_value = g->d_value;
   int rc = run_kernel(g, D, g->stream);
   if (rc) return rc;
@@ -108,6 +108,14 @@ mf_options with(const mf_options &o, Coord c, int k) {
 
 bool same(const mf_options &a, const mf_options &b) { return memcmp(&a, &b, sizeof(mf_options)) == 0; }
 
+// Whether g is solved in the same way with a and with b: as a lattice, by options
+// that differ only where a lattice solve reads none. Timing both would choose one
+// by noise.
+bool same_lattice_solve(const mf_graph *g, const mf_options &a, const mf_options &b) {
+  return lattice_applies(g, a) && lattice_applies(g, b) && a.gr_time_ratio == b.gr_time_ratio &&
+         (g->lat.dim == 3 || a.blocks_per_sm == b.blocks_per_sm);
+}
+
 }  // namespace
 
 // Replaces the options of g (validated; the launch shape is recomputed). On
@@ -148,7 +156,7 @@ int autotune(mf_graph *g, const mf_tune_spec *spec, mf_options *best, double *be
       for (int k = 0; k < candidates((Coord)c); k++) {
         if (budget > 0 && spent >= budget) goto done;
         const mf_options o = with(cur, (Coord)c, k);
-        if (same(o, cur)) continue;
+        if (same(o, cur) || same_lattice_solve(g, o, cur)) continue;
         // the local lists and BFS hops act only on graphs whose vertices are all thread-sized
         if ((c == LOCAL || c == HOPS) && keep_local_limit(o, g->max_degree, o.block_threads) == 0 &&
             keep_local_limit(cur, g->max_degree, cur.block_threads) == 0)

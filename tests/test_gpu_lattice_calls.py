@@ -111,6 +111,19 @@ def test_unions_of_one_are_not_prepared_as_lattices(gpu):
     assert abs(used[0] - used[1]) <= 8 << 20, used
 
 
+def test_autotune_of_a_lattice_moves_only_what_it_reads(gpu):
+    """Options that a lattice solve does not read are not tuned by the noise between identical solves."""
+    g = grid((300, 260), 4)
+    csr = gpu.build_csr(g.n, g.tail, g.head, g.cap)
+    start = gpu.default_options()
+    with gpu.Graph.from_csr(csr, g.s, g.t, start) as G:
+        value = G.solve(flow=False).value
+        best, ms = G.autotune(reps=1, sweeps=2)
+        assert G.solve(flow=False).value == value and on_lattice(G.stats())
+    d, s = gpu.options_to_dict(best), gpu.options_to_dict(start)
+    assert {k for k in d if d[k] != s[k]} <= {"gr_time_ratio", "blocks_per_sm"}
+
+
 @pytest.mark.parametrize("dims,lattice", [((2, 60000), True), ((2, 140000), False), ((40005, 8), True), ((40000, 7), False),
                                           ((4, 5, 20000), True), ((3, 4, 40000), False), ((200, 3), True)])
 def test_thin_boxes_take_the_faster_solver(gpu, dims, lattice):
