@@ -27,7 +27,7 @@ BUILD_LIMIT = os.path.join(PKG, "_build_limit")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 CU_SOURCES = ["mf_kernels_m0.cu", "mf_kernels_m1.cu", "mf_kernels_s0.cu", "mf_kernels_s1.cu", "mf_solver.cu", "mf_api.cu", "mf_batch.cu", "mf_service.cu", "mf_noalloc.cu", "mf_tune.cu", "mf_lattice.cu", "mf_lattice2.cu", "mf_lattice3.cu"]
 CPP_SOURCES = ["mf_csr.cpp"]
-HEADERS = ["mf_solver.cuh", "mf_lattice.cuh", "mf_tile_queue.cuh", "mf_device.cuh", "mf_internal.h"]
+HEADERS = ["mf_solver.cuh", "mf_lattice.cuh", "mf_check.cuh", "mf_tile_queue.cuh", "mf_device.cuh", "mf_internal.h"]
 
 
 def nvcc() -> str:

@@ -494,9 +494,12 @@ int device_status(const Ctl &c) {
                                 "discharge barrier", "apply barrier", "cut BFS (preflow)", "excess check",
                                 "phase-2 excess check", "cut BFS", "round limit", "list capacity",
                                 "settle barrier", "gap relabeling"};
-  if (c.err == MF_ERR_INTERNAL && c.err_where >= 1000)  // a build with gather checks (MF_CHECK_BOUNDS)
-    return fail(MF_ERR_INTERNAL, "gather index %lld out of bounds at mf_solver.cuh line %d", c.bad_index,
-                c.err_where - 1000);
+  static const char *check_files[] = {"mf_solver.cuh", "mf_lattice.cuh", "mf_lattice2.cu", "mf_lattice3.cu"};
+  if (c.err == MF_ERR_INTERNAL && c.err_where >= CHECK_WHERE) {  // a build with gather checks (MF_CHECK_BOUNDS)
+    const int at = c.err_where - CHECK_WHERE, file = at / CHECK_LINES;
+    return fail(MF_ERR_INTERNAL, "gather index %lld out of bounds at %s line %d", c.bad_index,
+                file < 4 ? check_files[file] : "?", at % CHECK_LINES);
+  }
   const char *w = (c.err_where >= 0 && c.err_where <= 13) ? where[c.err_where] : "?";
   if (c.err == MF_ERR_TIMEOUT) return fail(MF_ERR_TIMEOUT, "device wait timed out (%s)", w);
   if (c.err == MF_ERR_ITER_LIMIT) return fail(MF_ERR_ITER_LIMIT, "round limit reached (%lld rounds)", c.rounds);

@@ -13,6 +13,9 @@ constexpr int TILE_VERTICES = 1024;
 // carries UNV + 1 during a BFS so that it is never discovered.
 constexpr int UNV = 0x3fffffff;
 
+// err_where of an index check (mf_check.cuh): CHECK_WHERE + CHECK_LINES * file + line.
+constexpr int CHECK_WHERE = 1000, CHECK_LINES = 10000;
+
 // What the persistent kernel does.
 enum Mode : int {
   MODE_SOLVE = 0,   // phase 1, phase 2 (unless cut_only), cut, outputs

@@ -48,7 +48,11 @@
 #include <limits.h>
 
 #include "mf.h"
+#include "mf_check.cuh"
 #include "mf_device.cuh"
+
+#undef MF_FILE
+#define MF_FILE 1
 
 namespace mf {
 
@@ -209,12 +213,13 @@ __device__ __forceinline__ void start_relabel(const Dev &D, const int *drain, F 
       for (int k = lane; k < G::NH; k += 32) {
         const int j = k / G::FS, f = k % G::FS;
         if (!((bits >> j) & 1) || !G::face_entry(j, f)) continue;
-        const int a = __ldcg(&L.inbox[(size_t)t * G::NH + k]);
+        const int a = __ldcg(&L.inbox[MF_INBOX(D, (size_t)t * G::NH + k)]);
         if (a) {
           const int u = G::cell(j, f);
-          L.inbox[(size_t)t * G::NH + k] = 0;
-          L.r[((size_t)t * G::ND + j) * TV + u] = __ldcg(&L.r[((size_t)t * G::ND + j) * TV + u]) + a;
-          atomicAdd(reinterpret_cast<unsigned long long *>(&L.ex[(size_t)t * TV + u]), (unsigned long long)a);
+          L.inbox[MF_INBOX(D, (size_t)t * G::NH + k)] = 0;
+          int *const r = &L.r[MF_RES(D, ((size_t)t * G::ND + j) * TV + u)];
+          *r = __ldcg(r) + a;
+          atomicAdd(reinterpret_cast<unsigned long long *>(&L.ex[MF_CELL(D, (size_t)t * TV + u)]), (unsigned long long)a);
         }
       }
       __syncwarp();
@@ -222,15 +227,15 @@ __device__ __forceinline__ void start_relabel(const Dev &D, const int *drain, F 
 #pragma unroll 2
     for (int i = 0; i < TV / 128; i++) {
       const int u = 4 * (i * 32 + lane);
-      const int4 dr = __ldcg(reinterpret_cast<const int4 *>(&drain[(size_t)t * TV + u]));
+      const int4 dr = __ldcg(reinterpret_cast<const int4 *>(&drain[MF_CELL(D, (size_t)t * TV + u)]));
       unsigned m = 0;
 #pragma unroll
       for (int j = 0; j < G::ND; j++) {
-        const int4 r = __ldcg(reinterpret_cast<const int4 *>(&L.r[((size_t)t * G::ND + j) * TV + u]));
+        const int4 r = __ldcg(reinterpret_cast<const int4 *>(&L.r[MF_RES(D, ((size_t)t * G::ND + j) * TV + u)]));
         m |= ((unsigned)(r.x > 0) | (unsigned)(r.y > 0) << 8 | (unsigned)(r.z > 0) << 16 | (unsigned)(r.w > 0) << 24) << j;
       }
-      *reinterpret_cast<unsigned *>(&L.mask[(size_t)t * TV + u]) = m;
-      *reinterpret_cast<int4 *>(&L.d[(size_t)t * TV + u]) =
+      *reinterpret_cast<unsigned *>(&L.mask[MF_CELL(D, (size_t)t * TV + u)]) = m;
+      *reinterpret_cast<int4 *>(&L.d[MF_CELL(D, (size_t)t * TV + u)]) =
           make_int4(dr.x > 0 ? 1 : LINF, dr.y > 0 ? 1 : LINF, dr.z > 0 ? 1 : LINF, dr.w > 0 ? 1 : LINF);
       seed |= dr.x > 0 || dr.y > 0 || dr.z > 0 || dr.w > 0;
     }
@@ -250,8 +255,8 @@ __device__ __forceinline__ void queue_active(const Dev &D, F queue) {
 #pragma unroll 4
     for (int i = 0; i < TV / 64; i++) {
       const size_t at = (size_t)t * TV + 2 * (i * 32 + lane);
-      const longlong2 e = __ldcg(reinterpret_cast<const longlong2 *>(&L.ex[at]));
-      const int2 d = __ldcg(reinterpret_cast<const int2 *>(&L.d[at]));
+      const longlong2 e = __ldcg(reinterpret_cast<const longlong2 *>(&L.ex[MF_CELL(D, at)]));
+      const int2 d = __ldcg(reinterpret_cast<const int2 *>(&L.d[MF_CELL(D, at)]));
       a |= (e.x > 0 && d.x < LINF) || (e.y > 0 && d.y < LINF);
     }
     if (__any_sync(LFULL, a) && lane == 0) queue(t);
@@ -286,13 +291,13 @@ __device__ __forceinline__ long long start_cut(const Dev &D, F queue) {
           if (nt < 0) continue;
           q = (size_t)nt * TV + G::cell(j ^ 1, G::face(j, u));
         }
-        m |= ((__ldcg(&L.mask[q]) >> (j ^ 1)) & 1u) << j;
+        m |= ((__ldcg(&L.mask[MF_CELL(D, q)]) >> (j ^ 1)) & 1u) << j;
       }
-      const long long e = __ldcg(&L.ex[at]);
-      const bool sd = D.cut_only ? e > 0 : __ldcg(&L.ret[at]) != 0;
+      const long long e = __ldcg(&L.ex[MF_CELL(D, at)]);
+      const bool sd = D.cut_only ? e > 0 : __ldcg(&L.ret[MF_CELL(D, at)]) != 0;
       if (!D.cut_only && e != 0) left++;
-      L.ret[at] = (unsigned char)m;  // from here on the mask of the cut
-      L.d[at] = sd ? 0 : LINF;
+      L.ret[MF_CELL(D, at)] = (unsigned char)m;  // from here on the mask of the cut
+      L.d[MF_CELL(D, at)] = sd ? 0 : LINF;
       seed |= sd;
     }
     if (__syncthreads_or(seed) && threadIdx.x == 0) queue(t);
@@ -368,15 +373,15 @@ __device__ __forceinline__ void init_cells(const Dev &D) {
       for (int j = 0; j < G::ND; j++) r[j] = 0;
       if (p >= 0) {
         const int v = vertex_of(L, p);
-        const int b = __ldg(&D.row[v]), e = __ldg(&D.row[v + 1]);
+        const int b = __ldg(&D.row[MF_ROW(D, v)]), e = __ldg(&D.row[MF_ROW(D, v + 1)]);
         for (int a = b; a < e; a++) {
-          const int w = __ldg(&D.head[a]), cp = __ldg(&D.cap[a]);
+          const int w = __ldg(&D.head[MF_SLOT(D, a)]), cp = __ldg(&D.cap[MF_SLOT(D, a)]);
           if (w == L.t) {
             dr = cp;
             slots += 8;
           } else if (w == L.s) {
             slots += 16;
-            const int cs = __ldg(&D.cap[__ldg(&D.rev[a])]);
+            const int cs = __ldg(&D.cap[MF_SLOT(D, __ldg(&D.rev[MF_SLOT(D, a)]))]);
             rs = cp + cs;
             ex = cs;
           } else {
@@ -389,16 +394,16 @@ __device__ __forceinline__ void init_cells(const Dev &D) {
         }
       }
       const size_t at = (size_t)t * TV + u;
-      L.ex[at] = ex;
-      L.drain[at] = dr;
-      L.back[at] = rs;
-      L.ret[at] = 0;
-      if (DIM == 3) L.slots[at] = (unsigned char)slots;
+      L.ex[MF_CELL(D, at)] = ex;
+      L.drain[MF_CELL(D, at)] = dr;
+      L.back[MF_CELL(D, at)] = rs;
+      L.ret[MF_CELL(D, at)] = 0;
+      if (DIM == 3) L.slots[MF_CELL(D, at)] = (unsigned char)slots;
 #pragma unroll
-      for (int j = 0; j < G::ND; j++) L.r[((size_t)t * G::ND + j) * TV + u] = r[j];
+      for (int j = 0; j < G::ND; j++) L.r[MF_RES(D, ((size_t)t * G::ND + j) * TV + u)] = r[j];
     }
-    for (int k = threadIdx.x; k < G::NH; k += LT) L.inbox[(size_t)t * G::NH + k] = 0;
-    if (threadIdx.x == 0) L.state[t] = L.bits[t] = L.bits[(size_t)L.tiles + t] = 0;
+    for (int k = threadIdx.x; k < G::NH; k += LT) L.inbox[MF_INBOX(D, (size_t)t * G::NH + k)] = 0;
+    if (threadIdx.x == 0) L.state[MF_TILE(D, t)] = L.bits[MF_BITS(D, t)] = L.bits[MF_BITS(D, (size_t)L.tiles + t)] = 0;
   }
 }
 
@@ -413,7 +418,8 @@ __device__ __forceinline__ void write_outputs(const Dev &D) {
     const int words = (D.n + 31) >> 5, lane = threadIdx.x & 31;
     for (int wd = tid >> 5; wd < words; wd += nthr >> 5) {
       const int v = wd * 32 + lane;
-      const bool in = v < D.n && v != L.t && (v == L.s || __ldcg(&L.d[place_of<DIM>(L, cell_of(L, v))]) < LINF);
+      const bool in =
+          v < D.n && v != L.t && (v == L.s || __ldcg(&L.d[MF_CELL(D, place_of<DIM>(L, cell_of(L, v)))]) < LINF);
       const unsigned b = __ballot_sync(LFULL, in);
       if (lane == 0) D.out_cut[wd] = b;
     }
@@ -423,19 +429,19 @@ __device__ __forceinline__ void write_outputs(const Dev &D) {
       const int v = vertex_of(L, p);
       const size_t at = place_of<DIM>(L, p);
       const size_t rt = at / TV * G::ND * TV + at % TV;
-      const int b = __ldg(&D.row[v]), e = __ldg(&D.row[v + 1]);
+      const int b = __ldg(&D.row[MF_ROW(D, v)]), e = __ldg(&D.row[MF_ROW(D, v + 1)]);
       for (int a = b; a < e; a++) {
-        const int w = __ldg(&D.head[a]), cp = __ldg(&D.cap[a]);
+        const int w = __ldg(&D.head[MF_SLOT(D, a)]), cp = __ldg(&D.cap[MF_SLOT(D, a)]);
         if (w == L.t) {
-          D.out_flow[a] = cp - __ldcg(&L.drain[at]);
-          D.out_flow[__ldg(&D.rev[a])] = 0;
+          D.out_flow[MF_SLOT(D, a)] = cp - __ldcg(&L.drain[MF_CELL(D, at)]);
+          D.out_flow[MF_SLOT(D, __ldg(&D.rev[MF_SLOT(D, a)]))] = 0;
         } else if (w == L.s) {
-          const int net = __ldcg(&L.back[at]) - cp;  // flow s -> p
-          D.out_flow[a] = max(-net, 0);
-          D.out_flow[__ldg(&D.rev[a])] = max(net, 0);
+          const int net = __ldcg(&L.back[MF_CELL(D, at)]) - cp;  // flow s -> p
+          D.out_flow[MF_SLOT(D, a)] = max(-net, 0);
+          D.out_flow[MF_SLOT(D, __ldg(&D.rev[MF_SLOT(D, a)]))] = max(net, 0);
         } else {
-          const int res = __ldcg(&L.r[rt + (size_t)dir_of<DIM>(L, p, cell_of(L, w)) * TV]);
-          D.out_flow[a] = max(cp - res, 0);
+          const int res = __ldcg(&L.r[MF_RES(D, rt + (size_t)dir_of<DIM>(L, p, cell_of(L, w)) * TV)]);
+          D.out_flow[MF_SLOT(D, a)] = max(cp - res, 0);
         }
       }
     }

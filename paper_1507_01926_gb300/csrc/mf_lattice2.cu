@@ -9,6 +9,9 @@
 #include "mf_lattice.cuh"
 #include "mf_internal.h"
 
+#undef MF_FILE
+#define MF_FILE 2
+
 namespace mf {
 
 namespace {
@@ -27,10 +30,10 @@ struct CTile {
 
 // Queues tile t for sweep `sweep` (list generation gen), once.
 __device__ __forceinline__ void queue_tile(const Dev &D, int t, int sweep, int gen) {
-  if (atomicExch(&D.lat.state[t], sweep) != sweep) {
+  if (atomicExch(&D.lat.state[MF_TILE(D, t)], sweep) != sweep) {
     const int i = atomicAdd(&D.ctl->cnt[gen & 3], 1);
     if (i < D.lat.tiles)
-      D.lat.list[gen & 1][i] = t;
+      D.lat.list[gen & 1][MF_TILE(D, i)] = t;
     else
       lat_err(D, MF_ERR_INTERNAL, 11);
   }
@@ -53,7 +56,7 @@ __device__ __forceinline__ void for_tiles(const Dev &D, LShared &sh, int gen, in
   for (int i = blockIdx.x; i < n;) {
     int nx = 0;
     if (threadIdx.x == 0) nx = (int)gridDim.x + atomicAdd(&D.ctl->lcnt[gen & 3], 1);
-    f(__ldcg(&D.lat.list[gen & 1][i]));
+    f(__ldcg(&D.lat.list[gen & 1][MF_TILE(D, i)]));
     __syncthreads();  // the visit's shared state may be overwritten
     if (threadIdx.x == 0) sh.tick = nx;
     __syncthreads();
@@ -75,7 +78,8 @@ __device__ __forceinline__ void load_halo(const Dev &D, CTile<DIM> &w, int t) {
     const int st = j < 2 ? 1 : j < 4 ? L.TX : L.TX * L.TY;
     const bool there = up ? at + 1 < end : at > 0;
     const int n = up ? t + st : t - st;
-    w.lab[G::pad(G::cell(j, f)) + G::pstep(j)] = there ? __ldcg(&L.d[(size_t)n * TV + G::cell(j ^ 1, f)]) : LINF;
+    w.lab[MF_LAB(D, G::pad(G::cell(j, f)) + G::pstep(j))] =
+        there ? __ldcg(&L.d[MF_CELL(D, (size_t)n * TV + G::cell(j ^ 1, f))]) : LINF;
   }
 }
 
@@ -95,7 +99,7 @@ __device__ void push_visit(const Dev &D, CTile<DIM> &w, int t, int sweep, int ge
                            LStat &st) {
   using G = Geo<DIM>;
   const Lat &L = D.lat;
-  const int bits = __ldcg(&L.bits[(size_t)(sweep & 1) * L.tiles + t]);
+  const int bits = __ldcg(&L.bits[MF_BITS(D, (size_t)(sweep & 1) * L.tiles + t)]);
   int r[2][G::ND], d[2], dr[2];
   long long ex[2];
   unsigned in[2], ch = 0;  // directions that stay in the tile; bits c, 2 + c, 4 + c: residuals/excess, label, drain changed
@@ -104,10 +108,10 @@ __device__ void push_visit(const Dev &D, CTile<DIM> &w, int t, int sweep, int ge
     const int u = threadIdx.x + c * LT;
     const size_t at = (size_t)t * TV + u;
 #pragma unroll
-    for (int j = 0; j < G::ND; j++) r[c][j] = __ldcg(&L.r[((size_t)t * G::ND + j) * TV + u]);
-    ex[c] = __ldcg(&L.ex[at]);
-    d[c] = __ldcg(&L.d[at]);
-    dr[c] = __ldcg(&drain[at]);
+    for (int j = 0; j < G::ND; j++) r[c][j] = __ldcg(&L.r[MF_RES(D, ((size_t)t * G::ND + j) * TV + u)]);
+    ex[c] = __ldcg(&L.ex[MF_CELL(D, at)]);
+    d[c] = __ldcg(&L.d[MF_CELL(D, at)]);
+    dr[c] = __ldcg(&drain[MF_CELL(D, at)]);
     in[c] = 0;
 #pragma unroll
     for (int j = 0; j < G::ND; j++) in[c] |= (unsigned)G::inside(j, u) << j;
@@ -122,16 +126,17 @@ __device__ void push_visit(const Dev &D, CTile<DIM> &w, int t, int sweep, int ge
 #pragma unroll
       for (int j = 0; j < G::ND; j++)
         if ((bits >> j) & 1 & ~(in[c] >> j)) {
-          const int a = atomicExch(&L.inbox[(size_t)t * G::NH + j * G::FS + G::face(j, threadIdx.x + c * LT)], 0);
+          const int a =
+              atomicExch(&L.inbox[MF_INBOX(D, (size_t)t * G::NH + j * G::FS + G::face(j, threadIdx.x + c * LT))], 0);
           r[c][j] += a;
           ex[c] += a;
           ch |= 1u << c;
         }
   }
 #pragma unroll
-  for (int c = 0; c < 2; c++) w.lab[G::pad(threadIdx.x + c * LT)] = d[c];
+  for (int c = 0; c < 2; c++) w.lab[MF_LAB(D, G::pad(threadIdx.x + c * LT))] = d[c];
   __syncthreads();  // every thread has read the tile's bits
-  if (bits && threadIdx.x == 0) L.bits[(size_t)(sweep & 1) * L.tiles + t] = 0;
+  if (bits && threadIdx.x == 0) L.bits[MF_BITS(D, (size_t)(sweep & 1) * L.tiles + t)] = 0;
   const int cap = D.n_cap;
   unsigned outb = 0;
   for (int k = 0; k < LAT_ROUNDS; k++) {
@@ -145,7 +150,7 @@ __device__ void push_visit(const Dev &D, CTile<DIM> &w, int t, int sweep, int ge
       st.scans_dis += G::ND + 1;
       int dl[G::ND];
 #pragma unroll
-      for (int j = 0; j < G::ND; j++) dl[j] = w.lab[q + G::pstep(j)];
+      for (int j = 0; j < G::ND; j++) dl[j] = w.lab[MF_LAB(D, q + G::pstep(j))];
       int left = (int)min(ex[c], (long long)INT_MAX);
       ex[c] -= left;
       ch |= 1u << c;
@@ -156,7 +161,7 @@ __device__ void push_visit(const Dev &D, CTile<DIM> &w, int t, int sweep, int ge
         st.to_sink += a;
         st.pushes++;
         ch |= 16u << c;
-        if (ret) ret[(size_t)t * TV + u] = 0x80;
+        if (ret) ret[MF_CELL(D, (size_t)t * TV + u)] = 0x80;
       }
 #pragma unroll 1
       for (int pass = 0; left > 0; pass++) {
@@ -172,7 +177,7 @@ __device__ void push_visit(const Dev &D, CTile<DIM> &w, int t, int sweep, int ge
               w.delta[j][u] = a;
               atomicOr(&w.flag[u + G::step(j)], 1 << (j ^ 1));
             } else {
-              atomicAdd(&L.inbox[(size_t)w.nt[j] * G::NH + (j ^ 1) * G::FS + G::face(j, u)], a);
+              atomicAdd(&L.inbox[MF_INBOX(D, (size_t)w.nt[j] * G::NH + (j ^ 1) * G::FS + G::face(j, u))], a);
               outb |= 1u << j;
             }
           }
@@ -180,7 +185,7 @@ __device__ void push_visit(const Dev &D, CTile<DIM> &w, int t, int sweep, int ge
         }
         if (left == 0 || m + 1 <= d[c]) break;
         d[c] = min(m + 1, LINF);
-        w.lab[q] = d[c];
+        w.lab[MF_LAB(D, q)] = d[c];
         ch |= 4u << c;
         st.relabels++;
         if (pass || d[c] >= cap) break;
@@ -214,15 +219,15 @@ __device__ void push_visit(const Dev &D, CTile<DIM> &w, int t, int sweep, int ge
     const size_t at = (size_t)t * TV + u;
     if ((ch >> c) & 1) {
 #pragma unroll
-      for (int j = 0; j < G::ND; j++) L.r[((size_t)t * G::ND + j) * TV + u] = r[c][j];
-      L.ex[at] = ex[c];
+      for (int j = 0; j < G::ND; j++) L.r[MF_RES(D, ((size_t)t * G::ND + j) * TV + u)] = r[c][j];
+      L.ex[MF_CELL(D, at)] = ex[c];
     }
-    if ((ch >> (2 + c)) & 1) L.d[at] = d[c];
-    if ((ch >> (4 + c)) & 1) drain[at] = dr[c];
+    if ((ch >> (2 + c)) & 1) L.d[MF_CELL(D, at)] = d[c];
+    if ((ch >> (4 + c)) & 1) drain[MF_CELL(D, at)] = dr[c];
   }
   if (threadIdx.x < G::ND && ((w.out >> threadIdx.x) & 1)) {
     const int q = w.nt[threadIdx.x];
-    atomicOr(&L.bits[(size_t)((sweep + 1) & 1) * L.tiles + q], 1 << (threadIdx.x ^ 1));
+    atomicOr(&L.bits[MF_BITS(D, (size_t)((sweep + 1) & 1) * L.tiles + q)], 1 << (threadIdx.x ^ 1));
     queue_tile(D, q, sweep + 1, gen + 1);
   }
   if (threadIdx.x == 32 && act) queue_tile(D, t, sweep + 1, gen + 1);
@@ -241,14 +246,14 @@ __device__ void bfs_visit(const Dev &D, CTile<DIM> &w, int t, int sweep, int gen
 #pragma unroll
   for (int c = 0; c < 2; c++) {
     const size_t at = (size_t)t * TV + threadIdx.x + c * LT;
-    d0[c] = d[c] = __ldcg(&L.d[at]);
-    mk[c] = __ldcg(&mask[at]);
+    d0[c] = d[c] = __ldcg(&L.d[MF_CELL(D, at)]);
+    mk[c] = __ldcg(&mask[MF_CELL(D, at)]);
   }
   if (threadIdx.x < G::ND) w.nt[threadIdx.x] = next_tile<DIM>(L, t, threadIdx.x);
   load_halo<DIM>(D, w, t);
   if (threadIdx.x == 0) w.need = 0;
 #pragma unroll
-  for (int c = 0; c < 2; c++) w.lab[G::pad(threadIdx.x + c * LT)] = d[c];
+  for (int c = 0; c < 2; c++) w.lab[MF_LAB(D, G::pad(threadIdx.x + c * LT))] = d[c];
   __syncthreads();
   bool ch;
   do {
@@ -261,19 +266,19 @@ __device__ void bfs_visit(const Dev &D, CTile<DIM> &w, int t, int sweep, int gen
         int m = LINF;
 #pragma unroll
         for (int j = 0; j < G::ND; j++) {
-          const int x = *(volatile int *)&w.lab[q + G::pstep(j)];
+          const int x = *(volatile int *)&w.lab[MF_LAB(D, q + G::pstep(j))];
           if ((mk[c] >> j) & 1) m = min(m, x);
         }
         if (m + 1 < d[c]) {
           d[c] = m + 1;
-          *(volatile int *)&w.lab[q] = d[c];
+          *(volatile int *)&w.lab[MF_LAB(D, q)] = d[c];
           ch = true;
         }
       }
   } while (__syncthreads_or(ch));
 #pragma unroll
   for (int c = 0; c < 2; c++)
-    if (d[c] != d0[c]) L.d[(size_t)t * TV + threadIdx.x + c * LT] = d[c];
+    if (d[c] != d0[c]) L.d[MF_CELL(D, (size_t)t * TV + threadIdx.x + c * LT)] = d[c];
   st.scans_bfs += 2 * G::ND;
   st.visits_bfs += 2;
   unsigned need = 0;
@@ -282,8 +287,8 @@ __device__ void bfs_visit(const Dev &D, CTile<DIM> &w, int t, int sweep, int gen
     const int q = w.nt[j];
     if (q < 0 || !G::face_entry(j, f)) continue;
     const int at = G::pad(G::cell(j, f));
-    if (w.lab[at] + 1 < w.lab[at + G::pstep(j)] &&
-        ((__ldcg(&mask[(size_t)q * TV + G::cell(j ^ 1, f)]) >> (j ^ 1)) & 1))
+    if (w.lab[MF_LAB(D, at)] + 1 < w.lab[MF_LAB(D, at + G::pstep(j))] &&
+        ((__ldcg(&mask[MF_CELL(D, (size_t)q * TV + G::cell(j ^ 1, f))]) >> (j ^ 1)) & 1))
       need |= 1u << j;
   }
   if (need) atomicOr(&w.need, (int)need);
@@ -357,9 +362,10 @@ __global__ void __launch_bounds__(LT, 4) lattice2_kernel(Dev D) {
     }
     if (timer) D.ctl->grs++;
     start_relabel<DIM>(
-        D, drain, [&](int t) { return __ldcg(&L.bits[t]) | __ldcg(&L.bits[(size_t)L.tiles + t]); },
+        D, drain,
+        [&](int t) { return __ldcg(&L.bits[MF_BITS(D, t)]) | __ldcg(&L.bits[MF_BITS(D, (size_t)L.tiles + t)]); },
         [&](int t, bool seeds) {
-          L.bits[t] = L.bits[(size_t)L.tiles + t] = 0;
+          L.bits[MF_BITS(D, t)] = L.bits[MF_BITS(D, (size_t)L.tiles + t)] = 0;
           if (seeds) queue(t);
         });
     if (!next(2)) break;

@@ -16,6 +16,9 @@
 #include "mf_tile_queue.cuh"
 #include "mf_internal.h"
 
+#undef MF_FILE
+#define MF_FILE 3
+
 namespace mf {
 
 namespace {
@@ -171,7 +174,7 @@ static __device__ int q_pop(const Dev &D, LShared &sh, int ph, bool timed, bool 
 // (shifted by FACES), which the warp reads later with q_faces: the exchange is in
 // flight with the tile's loads.
 __device__ __forceinline__ int q_begin(const Dev &D, int ph, int t) {
-  return (threadIdx.x & 31) == 0 ? queue_of(D, ph).begin(t) : 0;
+  return (threadIdx.x & 31) == 0 ? queue_of(D, ph).begin(MF_TILE(D, t)) : 0;
 }
 __device__ __forceinline__ int q_faces(int old) {
   old = __shfl_sync(LFULL, old, 0);
@@ -190,9 +193,9 @@ __device__ __forceinline__ void q_done(const Dev &D, LTile<DIM> &w, int ph, unsi
   __threadfence();
   int put = -1;
   if (lane < Geo<DIM>::ND) {
-    if (((out >> lane) & 1) && q.mark(w.nt[lane], 1 << (lane ^ 1))) put = w.nt[lane];
+    if (((out >> lane) & 1) && q.mark(MF_TILE(D, w.nt[lane]), 1 << (lane ^ 1))) put = w.nt[lane];
   } else if (lane == 31) {
-    if (q.end(t, again)) put = t;
+    if (q.end(MF_TILE(D, t), again)) put = t;
   }
   __syncwarp();  // the pushes of all lanes together
   if (put >= 0) q.push(put, lane < 31);
@@ -215,26 +218,27 @@ __device__ __forceinline__ void load_labels(const Dev &D, LTile<DIM> &w, int t) 
   if (lane < G::ND) w.nt[lane] = nt;
   int4 own[4];
 #pragma unroll
-  for (int i = 0; i < 4; i++) own[i] = __ldcg(reinterpret_cast<const int4 *>(&L.d[(size_t)t * TV]) + i * 32 + lane);
+  for (int i = 0; i < 4; i++)
+    own[i] = __ldcg(reinterpret_cast<const int4 *>(&L.d[MF_CELL(D, (size_t)t * TV)]) + i * 32 + lane);
   int h[G::NH / 32];
 #pragma unroll
   for (int i = 0; i < G::NH / 32; i++) {
     const int j = i * 32 / G::FS, f = i * 32 % G::FS + lane, q = __shfl_sync(LFULL, nt, j);
     h[i] = LINF;
-    if (q >= 0 && G::face_entry(j, f)) h[i] = __ldcg(&L.d[(size_t)q * TV + G::cell(j ^ 1, f)]);
+    if (q >= 0 && G::face_entry(j, f)) h[i] = __ldcg(&L.d[MF_CELL(D, (size_t)q * TV + G::cell(j ^ 1, f))]);
   }
 #pragma unroll
   for (int i = 0; i < 4; i++) {  // four cells of one row
     const int p = G::pad(4 * (i * 32 + lane));
-    w.lab[p] = own[i].x;
-    w.lab[p + 1] = own[i].y;
-    w.lab[p + 2] = own[i].z;
-    w.lab[p + 3] = own[i].w;
+    w.lab[MF_LAB(D, p)] = own[i].x;
+    w.lab[MF_LAB(D, p + 1)] = own[i].y;
+    w.lab[MF_LAB(D, p + 2)] = own[i].z;
+    w.lab[MF_LAB(D, p + 3)] = own[i].w;
   }
 #pragma unroll
   for (int i = 0; i < G::NH / 32; i++) {
     const int j = i * 32 / G::FS, f = i * 32 % G::FS + lane;
-    if (G::face_entry(j, f)) w.lab[G::pad(G::cell(j, f)) + G::pstep(j)] = h[i];
+    if (G::face_entry(j, f)) w.lab[MF_LAB(D, G::pad(G::cell(j, f)) + G::pstep(j))] = h[i];
   }
 }
 
@@ -297,7 +301,7 @@ __device__ __forceinline__ int next_list(LTile<DIM> &w, unsigned &touched) {
 template <int DIM>
 __device__ __forceinline__ void push_out(const Dev &D, const LTile<DIM> &w, int j, int u, int a) {
   using G = Geo<DIM>;
-  atomicAdd(&D.lat.inbox[(size_t)w.nt[j] * G::NH + (j ^ 1) * G::FS + G::face(j, u)], a);
+  atomicAdd(&D.lat.inbox[MF_INBOX(D, (size_t)w.nt[j] * G::NH + (j ^ 1) * G::FS + G::face(j, u))], a);
 }
 
 // A round over the warp's list (n cells), 32 at a time, a lane per cell: every lane
@@ -319,13 +323,13 @@ __device__ __forceinline__ int push_round(const Dev &D, LTile<DIM> &w, int t, in
   for (int b = 0; b < n; b += 32) {
     const bool on = b + lane < n;
     const int u = w.q[on ? b + lane : 0], q = G::pad(u);
-    const int du = w.lab[q];
+    const int du = w.lab[MF_LAB(D, q)];
     long long e = 0;
     int left = 0, dr = 0;
     int r[G::ND], dl[G::ND];
 #pragma unroll
     for (int j = 0; j < G::ND; j++) {
-      dl[j] = w.lab[q + G::pstep(j)];
+      dl[j] = w.lab[MF_LAB(D, q + G::pstep(j))];
       r[j] = on ? w.r[j][u] : 0;
       st.scans_res += r[j] > 0;
     }
@@ -344,7 +348,7 @@ __device__ __forceinline__ int push_round(const Dev &D, LTile<DIM> &w, int t, in
         left -= a;
         st.to_sink += a;
         st.pushes++;
-        if (ret) ret[(size_t)t * TV + u] = 0x80;
+        if (ret) ret[MF_CELL(D, (size_t)t * TV + u)] = 0x80;
       }
     }
     __syncwarp();  // every lane has read its cell
@@ -380,7 +384,7 @@ __device__ __forceinline__ int push_round(const Dev &D, LTile<DIM> &w, int t, in
     if (on) {
       e += left;
       w.ex[u] = e;
-      if (lab != du) w.lab[q] = lab;
+      if (lab != du) w.lab[MF_LAB(D, q)] = lab;
       if (e > 0 && lab < cap) mark<DIM>(w, u);
     }
     __syncwarp();
@@ -405,12 +409,14 @@ __device__ void push_visit(const Dev &D, LTile<DIM> &w, int t, int ph, unsigned 
   const int state = q_begin(D, ph, t);
 #pragma unroll 4
   for (int i = 0; i < G::ND * TV / 128; i++)
-    copy16(&w.r[0][0] + 4 * (i * 32 + lane), &L.r[(size_t)t * G::ND * TV] + 4 * (i * 32 + lane));
+    copy16(&w.r[0][0] + 4 * (i * 32 + lane), &L.r[MF_RES(D, (size_t)t * G::ND * TV + 4 * (i * 32 + lane))]);
 #pragma unroll 4
-  for (int i = 0; i < TV / 64; i++) copy16(&w.ex[2 * (i * 32 + lane)], &L.ex[(size_t)t * TV + 2 * (i * 32 + lane)]);
+  for (int i = 0; i < TV / 64; i++)
+    copy16(&w.ex[2 * (i * 32 + lane)], &L.ex[MF_CELL(D, (size_t)t * TV + 2 * (i * 32 + lane))]);
 #pragma unroll
-  for (int i = 0; i < TV / 128; i++) copy16(&w.drain[4 * (i * 32 + lane)], &drain[(size_t)t * TV + 4 * (i * 32 + lane)]);
-  copy16(w.slots + 16 * lane, &L.slots[(size_t)t * TV + 16 * lane]);
+  for (int i = 0; i < TV / 128; i++)
+    copy16(&w.drain[4 * (i * 32 + lane)], &drain[MF_CELL(D, (size_t)t * TV + 4 * (i * 32 + lane))]);
+  copy16(w.slots + 16 * lane, &L.slots[MF_CELL(D, (size_t)t * TV + 16 * lane)]);
   load_labels<DIM>(D, w, t);  // (a halo older than the inbox is as good)
   const int bits = q_faces(state);
   if (bits) {
@@ -419,7 +425,8 @@ __device__ void push_visit(const Dev &D, LTile<DIM> &w, int t, int ph, unsigned 
     for (int i = 0; i < G::NH / 32; i++) {
       const int j = i * 32 / G::FS, f = i * 32 % G::FS + lane;
       a[i] = 0;
-      if (((bits >> j) & 1) && G::face_entry(j, f)) a[i] = atomicExch(&L.inbox[(size_t)t * G::NH + i * 32 + lane], 0);
+      if (((bits >> j) & 1) && G::face_entry(j, f))
+        a[i] = atomicExch(&L.inbox[MF_INBOX(D, (size_t)t * G::NH + i * 32 + lane)], 0);
     }
 #pragma unroll
     for (int i = 0; i < G::NH / 32; i++) w.got[i * 32 + lane] = a[i];
@@ -442,7 +449,7 @@ __device__ void push_visit(const Dev &D, LTile<DIM> &w, int t, int ph, unsigned 
   unsigned active = 0;
 #pragma unroll 4
   for (int i = 0; i < TV / 32; i++) {
-    const unsigned b = __ballot_sync(LFULL, w.ex[i * 32 + lane] > 0 && w.lab[G::pad(i * 32 + lane)] < cap);
+    const unsigned b = __ballot_sync(LFULL, w.ex[i * 32 + lane] > 0 && w.lab[MF_LAB(D, G::pad(i * 32 + lane))] < cap);
     if (lane == i) active = b;
   }
   if (lane < TV / 32) w.inq[lane] |= active;
@@ -459,10 +466,10 @@ __device__ void push_visit(const Dev &D, LTile<DIM> &w, int t, int ph, unsigned 
       const int u = i * 32 + lane;
       const size_t at = (size_t)t * TV + u;
 #pragma unroll
-      for (int j = 0; j < G::ND; j++) L.r[((size_t)t * G::ND + j) * TV + u] = w.r[j][u];
-      L.ex[at] = w.ex[u] + take<DIM>(w, u);
-      L.d[at] = w.lab[G::pad(u)];
-      drain[at] = w.drain[u];
+      for (int j = 0; j < G::ND; j++) L.r[MF_RES(D, ((size_t)t * G::ND + j) * TV + u)] = w.r[j][u];
+      L.ex[MF_CELL(D, at)] = w.ex[u] + take<DIM>(w, u);
+      L.d[MF_CELL(D, at)] = w.lab[MF_LAB(D, G::pad(u))];
+      drain[MF_CELL(D, at)] = w.drain[u];
     }
   }
   out = __reduce_or_sync(LFULL, out);
@@ -483,7 +490,7 @@ __device__ void bfs_visit(const Dev &D, LTile<DIM> &w, int t, int ph, const unsi
   const int lane = threadIdx.x & 31;
   unsigned char *mk = reinterpret_cast<unsigned char *>(w.ex);
   copy16(mk + 16 * lane, mask + (size_t)t * TV + 16 * lane);
-  copy16(w.slots + 16 * lane, &L.slots[(size_t)t * TV + 16 * lane]);
+  copy16(w.slots + 16 * lane, &L.slots[MF_CELL(D, (size_t)t * TV + 16 * lane)]);
   const int from = q_faces(q_begin(D, ph, t)), faces = from & 63;
   const bool seeds = from & (SEEDS >> FACES);
   load_labels<DIM>(D, w, t);
@@ -497,9 +504,9 @@ __device__ void bfs_visit(const Dev &D, LTile<DIM> &w, int t, int ph, const unsi
 #pragma unroll
     for (int f = lane; f < G::FS; f += 32) {
       if (!G::face_entry(j, f)) continue;
-      const int u = G::cell(j, f), q = G::pad(u), x = w.lab[q + G::pstep(j)] + 1;
-      if (((mk[u] >> j) & 1) && x < w.lab[q]) {  // one entry per cell and face
-        w.lab[q] = x;
+      const int u = G::cell(j, f), q = G::pad(u), x = w.lab[MF_LAB(D, q + G::pstep(j))] + 1;
+      if (((mk[u] >> j) & 1) && x < w.lab[MF_LAB(D, q)]) {  // one entry per cell and face
+        w.lab[MF_LAB(D, q)] = x;
         mark<DIM>(w, u);
       }
     }
@@ -511,7 +518,7 @@ __device__ void bfs_visit(const Dev &D, LTile<DIM> &w, int t, int ph, const unsi
 #pragma unroll 1
     for (int i = 0; i < TV / 32; i++) {
       const int u = i * 32 + lane;
-      put<DIM>(w, u, w.lab[G::pad(u)] < LINF, n);
+      put<DIM>(w, u, w.lab[MF_LAB(D, G::pad(u))] < LINF, n);
     }
     __syncwarp();
   }
@@ -519,18 +526,18 @@ __device__ void bfs_visit(const Dev &D, LTile<DIM> &w, int t, int ph, const unsi
     for (int b = 0; b < n; b += 32)
       if (b + lane < n) {
         const int u = w.q[b + lane], q = G::pad(u);
-        const int l = w.lab[q] + 1;
+        const int l = w.lab[MF_LAB(D, q)] + 1;
         int x[G::ND];
         unsigned k[G::ND];
 #pragma unroll
         for (int j = 0; j < G::ND; j++) {
-          x[j] = w.lab[q + G::pstep(j)];
+          x[j] = w.lab[MF_LAB(D, q + G::pstep(j))];
           k[j] = G::inside(j, u) ? mk[u + G::step(j)] : 0;
         }
 #pragma unroll
         for (int j = 0; j < G::ND; j++)
           if (((k[j] >> (j ^ 1)) & 1) && x[j] > l) {
-            atomicMin(&w.lab[q + G::pstep(j)], l);
+            atomicMin(&w.lab[MF_LAB(D, q + G::pstep(j))], l);
             mark<DIM>(w, u + G::step(j));
           }
         st.scans_bfs += w.slots[u] & 7;
@@ -542,7 +549,7 @@ __device__ void bfs_visit(const Dev &D, LTile<DIM> &w, int t, int ph, const unsi
 #pragma unroll 1
   for (int i = 0; i < TV / 32; i++) {
     const unsigned b = __shfl_sync(LFULL, touched, i);
-    if ((b >> lane) & 1) L.d[(size_t)t * TV + i * 32 + lane] = w.lab[G::pad(i * 32 + lane)];
+    if ((b >> lane) & 1) L.d[MF_CELL(D, (size_t)t * TV + i * 32 + lane)] = w.lab[MF_LAB(D, G::pad(i * 32 + lane))];
   }
   unsigned need = 0;
 #pragma unroll
@@ -550,8 +557,8 @@ __device__ void bfs_visit(const Dev &D, LTile<DIM> &w, int t, int ph, const unsi
     const int j = i * 32 / G::FS, f = i * 32 % G::FS + lane;
     const int at = G::face_entry(j, f) ? G::pad(G::cell(j, f)) : 0;
     // (a halo cell without a tile has label LINF and no arc)
-    if (G::face_entry(j, f) && w.nt[j] >= 0 && w.lab[at] + 1 < w.lab[at + G::pstep(j)])
-      need |= (unsigned)((__ldcg(&mask[(size_t)w.nt[j] * TV + G::cell(j ^ 1, f)]) >> (j ^ 1)) & 1) << j;
+    if (G::face_entry(j, f) && w.nt[j] >= 0 && w.lab[MF_LAB(D, at)] + 1 < w.lab[MF_LAB(D, at + G::pstep(j))])
+      need |= (unsigned)((__ldcg(&mask[MF_CELL(D, (size_t)w.nt[j] * TV + G::cell(j ^ 1, f))]) >> (j ^ 1)) & 1) << j;
   }
   need = __reduce_or_sync(LFULL, need);
   q_done<DIM>(D, w, ph, ~0ull, t, need, false);
@@ -589,7 +596,7 @@ __global__ void __launch_bounds__(LT, 1) lattice3_kernel(Dev D) {
     q_clear(D, ph);
     if (cutting) {
       const long long left = lat_sum(start_cut<DIM>(D, [&](int t) {
-        L.state[t] = QUEUED | SEEDS;
+        L.state[MF_TILE(D, t)] = QUEUED | SEEDS;
         queue_of(D, ph).push(t, false);
       }), sh.sum);
       if (threadIdx.x == 0 && left) {
@@ -599,9 +606,9 @@ __global__ void __launch_bounds__(LT, 1) lattice3_kernel(Dev D) {
     } else {
       if (timer) D.ctl->grs++;
       start_relabel<DIM>(
-          D, drain, [&](int t) { return __ldcg(&L.state[t]) >> FACES; },
+          D, drain, [&](int t) { return __ldcg(&L.state[MF_TILE(D, t)]) >> FACES; },
           [&](int t, bool seeds) {
-            L.state[t] = seeds ? QUEUED | SEEDS : 0;
+            L.state[MF_TILE(D, t)] = seeds ? QUEUED | SEEDS : 0;
             if (seeds) queue_of(D, ph).push(t, false);
           });
     }
@@ -614,7 +621,7 @@ __global__ void __launch_bounds__(LT, 1) lattice3_kernel(Dev D) {
     ph++;
     q_clear(D, ph);
     queue_active(D, [&](int t) {
-      L.state[t] = QUEUED;
+      L.state[MF_TILE(D, t)] = QUEUED;
       queue_of(D, ph).push(t, false);
     });
     ok = lat_sync(D, sh, 3);

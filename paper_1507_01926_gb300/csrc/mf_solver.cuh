@@ -50,7 +50,11 @@
 #include <stdint.h>
 
 #include "mf.h"
+#include "mf_check.cuh"
 #include "mf_device.cuh"
+
+#undef MF_FILE
+#define MF_FILE 0
 
 namespace cg = cooperative_groups;
 
@@ -82,32 +86,6 @@ __device__ __forceinline__ void red_release_add64(unsigned long long *p, unsigne
 }
 
 __device__ __forceinline__ int vol_read(const int *p) { return *(const volatile int *)p; }
-
-// Index checks of the gathers (a build with MF_CHECK_BOUNDS, for tests): an
-// index outside its array is recorded in the error word (MF_ERR_INTERNAL, the
-// solver source line in err_where and the index in bad_index, first one wins)
-// and replaced by 0, so the access stays inside the array and the solve ends
-// at its next grid barrier; no trap. Without MF_CHECK_BOUNDS the macros are the
-// index itself.
-#ifdef MF_CHECK_BOUNDS
-static __device__ __noinline__ long long mf_bad_index(const Dev &D, long long i, int line) {
-  if (atomicCAS(&D.ctl->err, 0, MF_ERR_INTERNAL) == 0) {
-    atomicExch(&D.ctl->err_where, 1000 + line);
-    atomicExch(reinterpret_cast<unsigned long long *>(&D.ctl->bad_index), (unsigned long long)i);
-  }
-  return 0;
-}
-#define MF_CHECKED(D, i, lim) \
-  (((unsigned long long)(long long)(i) < (unsigned long long)(long long)(lim)) ? (i)                     \
-                                                                              : (decltype((i) + 0))mf_bad_index(D, (i), __LINE__))
-#define MF_SLOT(D, a) MF_CHECKED(D, a, (D).m)
-#define MF_VTX(D, v) MF_CHECKED(D, v, (D).n)
-#define MF_ROW(D, v) MF_CHECKED(D, v, (D).n + 1)
-#else
-#define MF_SLOT(D, a) (a)
-#define MF_VTX(D, v) (v)
-#define MF_ROW(D, v) (v)
-#endif
 
 // label slot p / active stamp slot p of v
 __device__ __forceinline__ int *lab_ptr(const Dev &D, int v, int p) { return reinterpret_cast<int *>(D.vs + MF_VTX(D, v)) + 2 * p; }

@@ -222,3 +222,26 @@ def test_volume_scans_count_slots_that_exist(gpu, cut_only):
     assert st["scans_discharge"] <= 3 * st["visits_discharge"] + 4 * 16 * st["rounds"]  # 16 rounds a visit at most
     assert 0 < st["scans_discharge_residual"] <= st["scans_discharge"]
     assert st["scans_bfs"] <= 2.1 * st["visits_bfs"]
+
+
+@pytest.mark.parametrize("opts", [{}, dict(cut_only=1), dict(gr_time_ratio=1e-6)])
+@pytest.mark.parametrize("dims", [(40, 37), (17, 33), (400, 3), (20, 18, 12), (9, 17, 7), (3, 4, 60)])
+def test_checked_build_runs_the_lattice_kernels(gpu, dims, opts):
+    """The build with checked gathers solves lattices by the lattice kernels, and finds no index out of bounds."""
+    from paper_1507_01926_gb300 import build as mfbuild
+
+    g = grid(dims, 10)
+    csr = gpu.build_csr(g.n, g.tail, g.head, g.cap)
+    ref = oracle.maxflow(g.n, g.s, g.t, g.tail, g.head, g.cap, want_flow=False)
+    before = gpu.use_library(mfbuild.build(check=True))
+    try:
+        with gpu.Graph.from_csr(csr, g.s, g.t, gpu.default_options(**opts)) as G:
+            r = G.solve(flow=not opts.get("cut_only"))
+            assert on_lattice(G.stats())
+    finally:
+        gpu.use_library(before)
+    cut = gpu.cut_bits_to_bool(r.cut_bits, g.n)
+    assert r.value == ref["value"] and np.array_equal(cut, ref["cut"])
+    if r.flow is not None:
+        f = np.where(csr.arc_slot >= 0, r.flow[np.maximum(csr.arc_slot, 0)], 0).astype(np.int64)
+        assert not oracle.check_flow(g.n, g.s, g.t, g.tail, g.head, g.cap, f, r.value, cut)
