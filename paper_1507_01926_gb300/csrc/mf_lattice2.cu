@@ -296,14 +296,6 @@ __device__ void bfs_visit(const Dev &D, CTile<DIM> &w, int t, int sweep, int gen
   if (threadIdx.x < G::ND && ((w.need >> threadIdx.x) & 1)) queue_tile(D, w.nt[threadIdx.x], sweep + 1, gen + 1);
 }
 
-// False, with the error set, once a solve has taken LAT_EFFORT sweeps (the same
-// number in every CTA).
-__device__ __forceinline__ bool within_effort(const Dev &D, int sweep) {
-  if (sweep <= LAT_EFFORT) return true;
-  if (threadIdx.x == 0) lat_err(D, MF_ERR_ITER_LIMIT, 10);
-  return false;
-}
-
 // Relaxes labels from the tiles of list generation gen on; false after an error.
 template <int DIM>
 __device__ __forceinline__ bool bfs_sweeps(const Dev &D, LShared &sh, CTile<DIM> &w, int &sweep, int &gen,
@@ -314,7 +306,6 @@ __device__ __forceinline__ bool bfs_sweeps(const Dev &D, LShared &sh, CTile<DIM>
     if (!lat_sync(D, sh, 2, gen + 1)) return false;
     gen++;
     sweep++;
-    if (!within_effort(D, sweep)) return false;
   }
   return true;
 }
@@ -347,7 +338,7 @@ __global__ void __launch_bounds__(LT, 4) lattice2_kernel(Dev D) {
       ok = lat_sync(D, sh, where, gen + 1, sweep);
       gen++;
       sweep++;
-      return ok = ok && within_effort(D, sweep);
+      return ok;
     };
     clear_next(D, gen);
     if (cutting) {
@@ -389,6 +380,11 @@ __global__ void __launch_bounds__(LT, 4) lattice2_kernel(Dev D) {
     }
     do {
       rounds++;
+      if (sweep > LAT_EFFORT) {  // (here only: a relabel ends by itself, as labels only fall in it)
+        lat_err(D, MF_ERR_ITER_LIMIT, 10);
+        ok = false;
+        break;
+      }
       if (timer) {
         D.ctl->gr_req[sweep & 1] = (double)(lat_timer() - t1) > D.gr_time_ratio * (double)(t1 - t0);
         st.tiles_dis++;
