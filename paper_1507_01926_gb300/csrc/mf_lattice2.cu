@@ -16,12 +16,13 @@ namespace mf {
 
 namespace {
 
+constexpr int DIM = 2;
+using G = Geo<DIM>;
 constexpr int LAT_ROUNDS = 8;  // push-relabel rounds per visit of a tile (16: 5-15% slower, 32: 20-70%)
 
 // A CTA's tile.
-template <int DIM>
 struct CTile {
-  int lab[Geo<DIM>::PAD];  // labels with the halo
+  int lab[G::PAD];  // labels with the halo
   int delta[2 * DIM][TV];  // amount cell u pushed in direction j this round
   int flag[TV];            // directions from which cell u received this round
   int nt[2 * DIM];         // tiles across the faces (-1: none)
@@ -50,7 +51,7 @@ __device__ __forceinline__ void clear_next(const Dev &D, int gen) {
 // The tiles of list generation gen (n of them), one after another: the first
 // by block index, the rest by ticket (a visit takes between one and LAT_ROUNDS
 // rounds).
-template <int DIM, typename F>
+template <typename F>
 __device__ __forceinline__ void for_tiles(const Dev &D, LShared &sh, int gen, int n, F f) {
   clear_next(D, gen);
   for (int i = blockIdx.x; i < n;) {
@@ -65,17 +66,14 @@ __device__ __forceinline__ void for_tiles(const Dev &D, LShared &sh, int gen, in
 }
 
 // Labels of the cells across the tile's faces.
-template <int DIM>
-__device__ __forceinline__ void load_halo(const Dev &D, CTile<DIM> &w, int t) {
-  using G = Geo<DIM>;
+__device__ __forceinline__ void load_halo(const Dev &D, CTile &w, int t) {
   const Lat &L = D.lat;
-  const int tx = t % L.TX, q = t / L.TX, ty = q % L.TY, tz = q / L.TY;
+  const int tx = t % L.TX, ty = t / L.TX;
   for (int k = threadIdx.x; k < G::NH; k += LT) {
     const int j = k / G::FS, f = k % G::FS;
     if (!G::face_entry(j, f)) continue;
     const bool up = j & 1;
-    const int at = j < 2 ? tx : j < 4 ? ty : tz, end = j < 2 ? L.TX : j < 4 ? L.TY : L.TZ;
-    const int st = j < 2 ? 1 : j < 4 ? L.TX : L.TX * L.TY;
+    const int at = j < 2 ? tx : ty, end = j < 2 ? L.TX : L.TY, st = j < 2 ? 1 : L.TX;
     const bool there = up ? at + 1 < end : at > 0;
     const int n = up ? t + st : t - st;
     w.lab[MF_LAB(D, G::pad(G::cell(j, f)) + G::pstep(j))] =
@@ -94,10 +92,8 @@ __device__ __forceinline__ void load_halo(const Dev &D, CTile<DIM> &w, int t) {
 // the receiver, who adds it to its own registers after the CTA barrier. (With
 // residuals and 64-bit excess in shared memory, updated by the pusher, a round
 // was a chain of dependent shared-memory accesses and took 2 us instead of 1.)
-template <int DIM>
-__device__ void push_visit(const Dev &D, CTile<DIM> &w, int t, int sweep, int gen, int *drain, unsigned char *ret,
+__device__ void push_visit(const Dev &D, CTile &w, int t, int sweep, int gen, int *drain, unsigned char *ret,
                            LStat &st) {
-  using G = Geo<DIM>;
   const Lat &L = D.lat;
   const int bits = __ldcg(&L.bits[MF_BITS(D, (size_t)(sweep & 1) * L.tiles + t)]);
   int r[2][G::ND], d[2], dr[2];
@@ -118,7 +114,7 @@ __device__ void push_visit(const Dev &D, CTile<DIM> &w, int t, int sweep, int ge
     w.flag[u] = 0;
   }
   if (threadIdx.x < G::ND) w.nt[threadIdx.x] = next_tile<DIM>(L, t, threadIdx.x);
-  load_halo<DIM>(D, w, t);
+  load_halo(D, w, t);
   if (threadIdx.x == 0) w.out = 0;
   if (bits) {  // uniform in the CTA
 #pragma unroll
@@ -237,9 +233,7 @@ __device__ void push_visit(const Dev &D, CTile<DIM> &w, int t, int sweep, int ge
 // neighbours that a lowered face label can improve are queued. Bit j of `mask`:
 // the arc between the cell and its neighbour in direction j leads toward the
 // seeds (global relabel: the cell's residual; cut: the neighbour's).
-template <int DIM>
-__device__ void bfs_visit(const Dev &D, CTile<DIM> &w, int t, int sweep, int gen, const unsigned char *mask, LStat &st) {
-  using G = Geo<DIM>;
+__device__ void bfs_visit(const Dev &D, CTile &w, int t, int sweep, int gen, const unsigned char *mask, LStat &st) {
   const Lat &L = D.lat;
   int d0[2], d[2];
   unsigned mk[2];
@@ -250,7 +244,7 @@ __device__ void bfs_visit(const Dev &D, CTile<DIM> &w, int t, int sweep, int gen
     mk[c] = __ldcg(&mask[MF_CELL(D, at)]);
   }
   if (threadIdx.x < G::ND) w.nt[threadIdx.x] = next_tile<DIM>(L, t, threadIdx.x);
-  load_halo<DIM>(D, w, t);
+  load_halo(D, w, t);
   if (threadIdx.x == 0) w.need = 0;
 #pragma unroll
   for (int c = 0; c < 2; c++) w.lab[MF_LAB(D, G::pad(threadIdx.x + c * LT))] = d[c];
@@ -297,11 +291,10 @@ __device__ void bfs_visit(const Dev &D, CTile<DIM> &w, int t, int sweep, int gen
 }
 
 // Relaxes labels from the tiles of list generation gen on; false after an error.
-template <int DIM>
-__device__ __forceinline__ bool bfs_sweeps(const Dev &D, LShared &sh, CTile<DIM> &w, int &sweep, int &gen,
+__device__ __forceinline__ bool bfs_sweeps(const Dev &D, LShared &sh, CTile &w, int &sweep, int &gen,
                                            const unsigned char *mask, LStat &st) {
   while (sh.cnt > 0) {
-    for_tiles<DIM>(D, sh, gen, sh.cnt, [&](int t) { bfs_visit<DIM>(D, w, t, sweep, gen, mask, st); });
+    for_tiles(D, sh, gen, sh.cnt, [&](int t) { bfs_visit(D, w, t, sweep, gen, mask, st); });
     if (blockIdx.x == 0 && threadIdx.x == 0) st.tiles_bfs++;
     if (!lat_sync(D, sh, 2, gen + 1)) return false;
     gen++;
@@ -313,8 +306,7 @@ __device__ __forceinline__ bool bfs_sweeps(const Dev &D, LShared &sh, CTile<DIM>
 // Four CTAs per SM (64 registers): visits wait for memory first and for CTA
 // barriers after, so other tiles' visits have to fill both.
 __global__ void __launch_bounds__(LT, 4) lattice2_kernel(Dev D) {
-  constexpr int DIM = 2;
-  __shared__ CTile<DIM> w;
+  __shared__ CTile w;
   __shared__ LShared sh;
   const Lat &L = D.lat;
   LStat st;
@@ -348,7 +340,7 @@ __global__ void __launch_bounds__(LT, 4) lattice2_kernel(Dev D) {
         lat_err(D, MF_ERR_INTERNAL, 8);
       }
       if (!next(9)) break;
-      ok = bfs_sweeps<DIM>(D, sh, w, sweep, gen, L.ret, st);
+      ok = bfs_sweeps(D, sh, w, sweep, gen, L.ret, st);
       break;
     }
     if (timer) D.ctl->grs++;
@@ -360,7 +352,7 @@ __global__ void __launch_bounds__(LT, 4) lattice2_kernel(Dev D) {
           if (seeds) queue(t);
         });
     if (!next(2)) break;
-    if (!(ok = bfs_sweeps<DIM>(D, sh, w, sweep, gen, L.mask, st))) break;
+    if (!(ok = bfs_sweeps(D, sh, w, sweep, gen, L.mask, st))) break;
     clear_next(D, gen);
     queue_active(D, queue);
     if (!next(3)) break;
@@ -390,7 +382,7 @@ __global__ void __launch_bounds__(LT, 4) lattice2_kernel(Dev D) {
         st.tiles_dis++;
       }
       unsigned char *const ret = stage == 2 ? L.ret : nullptr;
-      for_tiles<DIM>(D, sh, gen, sh.cnt, [&](int t) { push_visit<DIM>(D, w, t, sweep, gen, drain, ret, st); });
+      for_tiles(D, sh, gen, sh.cnt, [&](int t) { push_visit(D, w, t, sweep, gen, drain, ret, st); });
     } while (next(4) && sh.cnt > 0 && !sh.req);
     if (timer) D.ctl->t_dis += lat_timer() - t1;
   }

@@ -5,7 +5,7 @@
 // on a few lanes. With a CTA per tile, nearly every warp has one active lane and
 // all of them wait at the CTA barriers (a round took 1.3 us, four tiles per SM); a
 // warp per tile runs the same round in 0.6 us, eight tiles per SM. A visit is
-// about 16 us: 4 us to load 25 KB and take in the inboxes, ten rounds, 2.5 us to
+// about 16 us: 4 us to load 22 KB and take in the inboxes, ten rounds, 2.5 us to
 // write the touched cells back and hand on to the neighbours. A scheduler issues
 // an instruction every 8 cycles; of a warp's time a quarter is waiting for a tile
 // (97x80x61 has fewer active tiles than the GPU has warps), a quarter loads, a
@@ -23,19 +23,20 @@ namespace mf {
 
 namespace {
 
+constexpr int DIM = 3;
+using G = Geo<DIM>;
 constexpr int LAT_ROUNDS = 16;  // push-relabel rounds per visit of a tile (8 and 32 measured 3-8% slower)
 
 // A warp's tile.
-template <int DIM>
 struct __align__(16) LTile {
   int r[2 * DIM][TV];
   long long ex[TV];
   int drain[TV];
-  int lab[Geo<DIM>::PAD];  // labels with the halo
+  int lab[G::PAD];  // labels with the halo
   unsigned lo[TV], hi[TV]; // excess received and not taken in yet: sums of the low 16 bits and of the rest
   union {
     unsigned short q[TV];    // the cells of this round
-    int got[Geo<DIM>::NH];   // while loading: amounts from the inbox, by face entry
+    int got[G::NH];   // while loading: amounts from the inbox, by face entry
   };
   __align__(16) unsigned char slots[TV];  // Lat::slots
   unsigned inq[TV / 32];   // bitmap of the cells of the next round
@@ -184,15 +185,14 @@ __device__ __forceinline__ int q_faces(int old) {
 
 // Ends the visit of tile t: the tiles across the faces in `out` have work now, and
 // t itself if `again`. All lanes; the warp's writes are released first.
-template <int DIM>
-__device__ __forceinline__ void q_done(const Dev &D, LTile<DIM> &w, int ph, unsigned long long deadline, int t, unsigned out,
+__device__ __forceinline__ void q_done(const Dev &D, LTile &w, int ph, unsigned long long deadline, int t, unsigned out,
                                        bool again) {
   const int lane = threadIdx.x & 31;
   TileQueue<QMem> q = queue_of(D, ph, deadline);
   __syncwarp();  // also: the warp's tile may be overwritten
   __threadfence();
   int put = -1;
-  if (lane < Geo<DIM>::ND) {
+  if (lane < G::ND) {
     if (((out >> lane) & 1) && q.mark(MF_TILE(D, w.nt[lane]), 1 << (lane ^ 1))) put = w.nt[lane];
   } else if (lane == 31) {
     if (q.end(MF_TILE(D, t), again)) put = t;
@@ -209,9 +209,7 @@ __device__ __forceinline__ void copy16(void *dst, const void *src) {
 
 // Labels of tile t and of the cells across its faces, into w.lab, and the tiles
 // across its faces, into w.nt (the caller synchronises the warp).
-template <int DIM>
-__device__ __forceinline__ void load_labels(const Dev &D, LTile<DIM> &w, int t) {
-  using G = Geo<DIM>;
+__device__ __forceinline__ void load_labels(const Dev &D, LTile &w, int t) {
   const Lat &L = D.lat;
   const int lane = threadIdx.x & 31;
   const int nt = next_tile<DIM>(L, t, lane);
@@ -225,7 +223,7 @@ __device__ __forceinline__ void load_labels(const Dev &D, LTile<DIM> &w, int t) 
   for (int i = 0; i < G::NH / 32; i++) {
     const int j = i * 32 / G::FS, f = i * 32 % G::FS + lane, q = __shfl_sync(LFULL, nt, j);
     h[i] = LINF;
-    if (q >= 0 && G::face_entry(j, f)) h[i] = __ldcg(&L.d[MF_CELL(D, (size_t)q * TV + G::cell(j ^ 1, f))]);
+    if (q >= 0) h[i] = __ldcg(&L.d[MF_CELL(D, (size_t)q * TV + G::cell(j ^ 1, f))]);
   }
 #pragma unroll
   for (int i = 0; i < 4; i++) {  // four cells of one row
@@ -238,19 +236,17 @@ __device__ __forceinline__ void load_labels(const Dev &D, LTile<DIM> &w, int t) 
 #pragma unroll
   for (int i = 0; i < G::NH / 32; i++) {
     const int j = i * 32 / G::FS, f = i * 32 % G::FS + lane;
-    if (G::face_entry(j, f)) w.lab[MF_LAB(D, G::pad(G::cell(j, f)) + G::pstep(j))] = h[i];
+    w.lab[MF_LAB(D, G::pad(G::cell(j, f)) + G::pstep(j))] = h[i];
   }
 }
 
 // Marks cell u for the next list.
-template <int DIM>
-__device__ __forceinline__ void mark(LTile<DIM> &w, int u) {
+__device__ __forceinline__ void mark(LTile &w, int u) {
   atomicOr(&w.inq[u >> 5], 1u << (u & 31));
 }
 
 // Appends one cell of every lane with `on` to the list of n cells.
-template <int DIM>
-__device__ __forceinline__ void put(LTile<DIM> &w, int u, bool on, int &n) {
+__device__ __forceinline__ void put(LTile &w, int u, bool on, int &n) {
   const unsigned b = __ballot_sync(LFULL, on);
   if (on) w.q[n + __popc(b & ((1u << (threadIdx.x & 31)) - 1))] = (unsigned short)u;
   n += __popc(b);
@@ -258,15 +254,13 @@ __device__ __forceinline__ void put(LTile<DIM> &w, int u, bool on, int &n) {
 
 // Adds a to the excess cell u receives: two 32-bit sums that 6 arcs cannot
 // overflow (a 64-bit add to shared memory is a compare-and-swap loop).
-template <int DIM>
-__device__ __forceinline__ void give(LTile<DIM> &w, int u, int a) {
+__device__ __forceinline__ void give(LTile &w, int u, int a) {
   atomicAdd(&w.lo[u], (unsigned)a & 0xffffu);
   atomicAdd(&w.hi[u], (unsigned)a >> 16);
 }
 
 // Takes what cell u received.
-template <int DIM>
-__device__ __forceinline__ long long take(LTile<DIM> &w, int u) {
+__device__ __forceinline__ long long take(LTile &w, int u) {
   const unsigned l = w.lo[u], h = w.hi[u];
   w.lo[u] = 0;
   w.hi[u] = 0;
@@ -276,8 +270,7 @@ __device__ __forceinline__ long long take(LTile<DIM> &w, int u) {
 // The marked cells become the warp's list (their number is returned, in every
 // lane), join `touched` (lane i < 16: cells 32 i to 32 i + 31), and the marks are
 // cleared.
-template <int DIM>
-__device__ __forceinline__ int next_list(LTile<DIM> &w, unsigned &touched) {
+__device__ __forceinline__ int next_list(LTile &w, unsigned &touched) {
   const int lane = threadIdx.x & 31;
   __syncwarp();
   unsigned x = lane < TV / 32 ? w.inq[lane] : 0;
@@ -298,9 +291,7 @@ __device__ __forceinline__ int next_list(LTile<DIM> &w, unsigned &touched) {
 }
 
 // A push over face j: the amount joins the inbox of the tile across it.
-template <int DIM>
-__device__ __forceinline__ void push_out(const Dev &D, const LTile<DIM> &w, int j, int u, int a) {
-  using G = Geo<DIM>;
+__device__ __forceinline__ void push_out(const Dev &D, const LTile &w, int j, int u, int a) {
   atomicAdd(&D.lat.inbox[MF_INBOX(D, (size_t)w.nt[j] * G::NH + (j ^ 1) * G::FS + G::face(j, u))], a);
 }
 
@@ -315,10 +306,8 @@ __device__ __forceinline__ void push_out(const Dev &D, const LTile<DIM> &w, int 
 // which costs detours, not correctness). Nothing waits for an atomic's result: what
 // a cell received and whether it is active next are sums and bits read in the next
 // round.
-template <int DIM>
-__device__ __forceinline__ int push_round(const Dev &D, LTile<DIM> &w, int t, int n, unsigned char *ret, unsigned &out,
+__device__ __forceinline__ int push_round(const Dev &D, LTile &w, int t, int n, unsigned char *ret, unsigned &out,
                                           unsigned &touched, LStat &st) {
-  using G = Geo<DIM>;
   const int lane = threadIdx.x & 31, cap = D.n_cap;
   for (int b = 0; b < n; b += 32) {
     const bool on = b + lane < n;
@@ -334,7 +323,7 @@ __device__ __forceinline__ int push_round(const Dev &D, LTile<DIM> &w, int t, in
       st.scans_res += r[j] > 0;
     }
     if (on) {
-      e = w.ex[u] + take<DIM>(w, u);
+      e = w.ex[u] + take(w, u);
       // at most INT_MAX leaves a cell per round, so the chain of pushes is 32-bit
       left = du < cap ? (int)min(e, (long long)INT_MAX) : 0;
       e -= left;
@@ -373,10 +362,10 @@ __device__ __forceinline__ int push_round(const Dev &D, LTile<DIM> &w, int t, in
         if (G::inside(j, u)) {
           const int x = u + G::step(j);
           atomicAdd(&w.r[j ^ 1][x], a);
-          give<DIM>(w, x, a);
-          mark<DIM>(w, x);
+          give(w, x, a);
+          mark(w, x);
         } else {
-          push_out<DIM>(D, w, j, u, a);
+          push_out(D, w, j, u, a);
           out |= 1u << j;
         }
       }
@@ -385,11 +374,11 @@ __device__ __forceinline__ int push_round(const Dev &D, LTile<DIM> &w, int t, in
       e += left;
       w.ex[u] = e;
       if (lab != du) w.lab[MF_LAB(D, q)] = lab;
-      if (e > 0 && lab < cap) mark<DIM>(w, u);
+      if (e > 0 && lab < cap) mark(w, u);
     }
     __syncwarp();
   }
-  return next_list<DIM>(w, touched);
+  return next_list(w, touched);
 }
 
 // One visit of an active tile in phase `ph` by a warp: load, inboxes, rounds,
@@ -400,10 +389,8 @@ __device__ __forceinline__ int push_round(const Dev &D, LTile<DIM> &w, int t, in
 // On a volume about 1% of the cells of an active tile are active in a round: with
 // a CTA per tile and two cells per thread, nearly every warp had one active lane
 // and a round took 1.3 us.
-template <int DIM>
-__device__ void push_visit(const Dev &D, LTile<DIM> &w, int t, int ph, unsigned long long deadline, int *drain,
+__device__ void push_visit(const Dev &D, LTile &w, int t, int ph, unsigned long long deadline, int *drain,
                            unsigned char *ret, LStat &st) {
-  using G = Geo<DIM>;
   const Lat &L = D.lat;
   const int lane = threadIdx.x & 31, cap = D.n_cap;
   const int state = q_begin(D, ph, t);
@@ -417,16 +404,15 @@ __device__ void push_visit(const Dev &D, LTile<DIM> &w, int t, int ph, unsigned 
   for (int i = 0; i < TV / 128; i++)
     copy16(&w.drain[4 * (i * 32 + lane)], &drain[MF_CELL(D, (size_t)t * TV + 4 * (i * 32 + lane))]);
   copy16(w.slots + 16 * lane, &L.slots[MF_CELL(D, (size_t)t * TV + 16 * lane)]);
-  load_labels<DIM>(D, w, t);  // (a halo older than the inbox is as good)
+  load_labels(D, w, t);  // (a halo older than the inbox is as good)
   const int bits = q_faces(state);
   if (bits) {
     int a[G::NH / 32];
 #pragma unroll
     for (int i = 0; i < G::NH / 32; i++) {
-      const int j = i * 32 / G::FS, f = i * 32 % G::FS + lane;
+      const int j = i * 32 / G::FS;
       a[i] = 0;
-      if (((bits >> j) & 1) && G::face_entry(j, f))
-        a[i] = atomicExch(&L.inbox[MF_INBOX(D, (size_t)t * G::NH + i * 32 + lane)], 0);
+      if ((bits >> j) & 1) a[i] = atomicExch(&L.inbox[MF_INBOX(D, (size_t)t * G::NH + i * 32 + lane)], 0);
     }
 #pragma unroll
     for (int i = 0; i < G::NH / 32; i++) w.got[i * 32 + lane] = a[i];
@@ -440,8 +426,8 @@ __device__ void push_visit(const Dev &D, LTile<DIM> &w, int t, int ph, unsigned 
       if (a) {
         const int j = k / G::FS, u = G::cell(j, k % G::FS);
         w.r[j][u] += a;  // one entry per (face, cell)
-        give<DIM>(w, u, a);
-        mark<DIM>(w, u);
+        give(w, u, a);
+        mark(w, u);
       }
     }
     __syncwarp();
@@ -454,9 +440,9 @@ __device__ void push_visit(const Dev &D, LTile<DIM> &w, int t, int ph, unsigned 
   }
   if (lane < TV / 32) w.inq[lane] |= active;
   unsigned out = 0, touched = 0;  // lane i of touched: cells 32 i ... 32 i + 31 to be written back
-  int n = next_list<DIM>(w, touched);
+  int n = next_list(w, touched);
   for (int k = 0; k < LAT_ROUNDS && n > 0; k++) {
-    n = push_round<DIM>(D, w, t, n, ret, out, touched, st);
+    n = push_round(D, w, t, n, ret, out, touched, st);
   }
   __syncwarp();
 #pragma unroll 1
@@ -467,13 +453,13 @@ __device__ void push_visit(const Dev &D, LTile<DIM> &w, int t, int ph, unsigned 
       const size_t at = (size_t)t * TV + u;
 #pragma unroll
       for (int j = 0; j < G::ND; j++) L.r[MF_RES(D, ((size_t)t * G::ND + j) * TV + u)] = w.r[j][u];
-      L.ex[MF_CELL(D, at)] = w.ex[u] + take<DIM>(w, u);
+      L.ex[MF_CELL(D, at)] = w.ex[u] + take(w, u);
       L.d[MF_CELL(D, at)] = w.lab[MF_LAB(D, G::pad(u))];
       drain[MF_CELL(D, at)] = w.drain[u];
     }
   }
   out = __reduce_or_sync(LFULL, out);
-  q_done<DIM>(D, w, ph, deadline, t, out, n > 0);
+  q_done(D, w, ph, deadline, t, out, n > 0);
   st.tiles_dis += lane == 0;
 }
 
@@ -483,9 +469,7 @@ __device__ void push_visit(const Dev &D, LTile<DIM> &w, int t, int ph, unsigned 
 // queued. Bit j of `mask`: the arc between the cell and its neighbour in
 // direction j leads toward the seeds (global relabel: the cell's residual; cut:
 // the neighbour's).
-template <int DIM>
-__device__ void bfs_visit(const Dev &D, LTile<DIM> &w, int t, int ph, const unsigned char *mask, LStat &st) {
-  using G = Geo<DIM>;
+__device__ void bfs_visit(const Dev &D, LTile &w, int t, int ph, const unsigned char *mask, LStat &st) {
   const Lat &L = D.lat;
   const int lane = threadIdx.x & 31;
   unsigned char *mk = reinterpret_cast<unsigned char *>(w.ex);
@@ -493,7 +477,7 @@ __device__ void bfs_visit(const Dev &D, LTile<DIM> &w, int t, int ph, const unsi
   copy16(w.slots + 16 * lane, &L.slots[MF_CELL(D, (size_t)t * TV + 16 * lane)]);
   const int from = q_faces(q_begin(D, ph, t)), faces = from & 63;
   const bool seeds = from & (SEEDS >> FACES);
-  load_labels<DIM>(D, w, t);
+  load_labels(D, w, t);
   asm volatile("cp.async.wait_all;" ::: "memory");
   __syncwarp();
   int n = 0;
@@ -503,22 +487,21 @@ __device__ void bfs_visit(const Dev &D, LTile<DIM> &w, int t, int ph, const unsi
     const int j = __ffs(f6) - 1;
 #pragma unroll
     for (int f = lane; f < G::FS; f += 32) {
-      if (!G::face_entry(j, f)) continue;
       const int u = G::cell(j, f), q = G::pad(u), x = w.lab[MF_LAB(D, q + G::pstep(j))] + 1;
       if (((mk[u] >> j) & 1) && x < w.lab[MF_LAB(D, q)]) {  // one entry per cell and face
         w.lab[MF_LAB(D, q)] = x;
-        mark<DIM>(w, u);
+        mark(w, u);
       }
     }
     __syncwarp();
   }
-  n = next_list<DIM>(w, touched);
+  n = next_list(w, touched);
   if (seeds) {  // first visit: every cell with a label offers it
     n = 0;
 #pragma unroll 1
     for (int i = 0; i < TV / 32; i++) {
       const int u = i * 32 + lane;
-      put<DIM>(w, u, w.lab[MF_LAB(D, G::pad(u))] < LINF, n);
+      put(w, u, w.lab[MF_LAB(D, G::pad(u))] < LINF, n);
     }
     __syncwarp();
   }
@@ -538,12 +521,12 @@ __device__ void bfs_visit(const Dev &D, LTile<DIM> &w, int t, int ph, const unsi
         for (int j = 0; j < G::ND; j++)
           if (((k[j] >> (j ^ 1)) & 1) && x[j] > l) {
             atomicMin(&w.lab[MF_LAB(D, q + G::pstep(j))], l);
-            mark<DIM>(w, u + G::step(j));
+            mark(w, u + G::step(j));
           }
         st.scans_bfs += w.slots[u] & 7;
         st.visits_bfs++;
       }
-    n = next_list<DIM>(w, touched);
+    n = next_list(w, touched);
   }
   __syncwarp();
 #pragma unroll 1
@@ -555,22 +538,21 @@ __device__ void bfs_visit(const Dev &D, LTile<DIM> &w, int t, int ph, const unsi
 #pragma unroll
   for (int i = 0; i < G::NH / 32; i++) {
     const int j = i * 32 / G::FS, f = i * 32 % G::FS + lane;
-    const int at = G::face_entry(j, f) ? G::pad(G::cell(j, f)) : 0;
+    const int at = G::pad(G::cell(j, f));
     // (a halo cell without a tile has label LINF and no arc)
-    if (G::face_entry(j, f) && w.nt[j] >= 0 && w.lab[MF_LAB(D, at)] + 1 < w.lab[MF_LAB(D, at + G::pstep(j))])
+    if (w.nt[j] >= 0 && w.lab[MF_LAB(D, at)] + 1 < w.lab[MF_LAB(D, at + G::pstep(j))])
       need |= (unsigned)((__ldcg(&mask[MF_CELL(D, (size_t)w.nt[j] * TV + G::cell(j ^ 1, f))]) >> (j ^ 1)) & 1) << j;
   }
   need = __reduce_or_sync(LFULL, need);
-  q_done<DIM>(D, w, ph, ~0ull, t, need, false);
+  q_done(D, w, ph, ~0ull, t, need, false);
   st.tiles_bfs += lane == 0;
 }
 
-// One CTA of 8 warps per SM, a tile (25 KB) per warp.
+// One CTA of 8 warps per SM, a tile (28 KB) per warp.
 __global__ void __launch_bounds__(LT, 1) lattice3_kernel(Dev D) {
-  constexpr int DIM = 3;
   extern __shared__ __align__(16) unsigned char lat_smem[];
   __shared__ LShared sh;
-  LTile<DIM> &w = reinterpret_cast<LTile<DIM> *>(lat_smem)[threadIdx.x >> 5];
+  LTile &w = reinterpret_cast<LTile *>(lat_smem)[threadIdx.x >> 5];
   const Lat &L = D.lat;
   const int tid = blockIdx.x * LT + threadIdx.x, nthr = gridDim.x * LT;
   LStat st;
@@ -615,7 +597,7 @@ __global__ void __launch_bounds__(LT, 1) lattice3_kernel(Dev D) {
     ok = lat_sync(D, sh, 2);
     if (!ok) break;
     const unsigned char *const mask = cutting ? L.ret : L.mask;
-    for (int t; (t = q_pop(D, sh, ph, false, false, st)) >= 0;) bfs_visit<DIM>(D, w, t, ph, mask, st);
+    for (int t; (t = q_pop(D, sh, ph, false, false, st)) >= 0;) bfs_visit(D, w, t, ph, mask, st);
     ok = lat_sync(D, sh, cutting ? 9 : 2);
     if (!ok || cutting) break;
     ph++;
@@ -645,7 +627,7 @@ __global__ void __launch_bounds__(LT, 1) lattice3_kernel(Dev D) {
     __syncthreads();
     unsigned char *const ret = stage == 2 ? L.ret : nullptr;
     bool first = true;
-    for (int t; (t = q_pop(D, sh, ph, true, first, st)) >= 0; first = false) push_visit<DIM>(D, w, t, ph, sh.deadline, drain, ret, st);
+    for (int t; (t = q_pop(D, sh, ph, true, first, st)) >= 0; first = false) push_visit(D, w, t, ph, sh.deadline, drain, ret, st);
     ok = lat_sync(D, sh, 4);
     if (timer) D.ctl->t_dis += lat_timer() - t1;
   }
@@ -661,6 +643,6 @@ const void *lattice3_fn() { return (const void *)lattice3_kernel; }
 size_t lattice_queue_bytes(int tiles) {
   return (size_t)q_slots(tiles) * Q_STRIDE * 4;
 }
-size_t lattice3_smem() { return LW * sizeof(LTile<3>); }
+size_t lattice3_smem() { return LW * sizeof(LTile); }
 
 }  // namespace mf
