@@ -30,7 +30,8 @@
  * cells of a row-major 2D or 3D box, with arcs between neighbouring cells and
  * between cells and s or t only (at most one slot per direction and terminal,
  * found when the graph is created), is solved by mf_solve / mf_solve_device on
- * tiles of cells instead of vertex lists, where its options ask for nothing
+ * tiles of cells instead of vertex lists (large boxes so thin that their tiles
+ * would be mostly padding excepted), where its options ask for nothing
  * that only the list solver has: simple_rounds, gap_every and max_rounds 0,
  * gr_time_ratio > 0, block_threads 256, kernel_variant 0, local_lists on. Of the
  * options it then takes gr_time_ratio (its only relabel trigger), cut_only,

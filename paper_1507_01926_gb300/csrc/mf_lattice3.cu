@@ -11,7 +11,7 @@
 // (97x80x61 has fewer active tiles than the GPU has warps), a quarter loads, a
 // third the dependent instructions and branches of the rounds.
 // Measured, solve of 97x80x61 / 256x256x128: list solver 96 / 870 ms, a CTA per
-// tile in sweeps 30 / 750 ms, this 30 / 415 ms.
+// tile in sweeps 30 / 750 ms, this 33-41 / 375-480 ms by input.
 #include "mf_lattice.cuh"
 #include "mf_tile_queue.cuh"
 #include "mf_internal.h"

@@ -18,7 +18,8 @@ def extra(g, tail, head):
 
 def arc(g, what):
     inner = np.flatnonzero((g.tail != g.s) & (g.head != g.t) & (g.tail != g.t) & (g.head != g.s))[0]
-    return {"parallel arc": (g.tail[inner], g.head[inner]), "s-t arc": (g.s, g.t), "far arc": (0, g.n - 3)}[what]
+    width = {"grid2d": 80, "grid3d": 40}[g.name[:6]]  # cells in a row of GRIDS
+    return {"wrap": (width - 1, width), "parallel arc": (g.tail[inner], g.head[inner]), "s-t arc": (g.s, g.t), "far arc": (0, g.n - 3)}[what]
 
 
 def solve_and_check(mf, g, lattice, **opts):
@@ -45,7 +46,7 @@ def test_default_lists_on_grids(gpu, which, opts):
     solve_and_check(gpu, extra(g, *arc(g, "parallel arc")), False, **opts)
 
 
-@pytest.mark.parametrize("what", ["parallel arc", "s-t arc", "far arc"])
+@pytest.mark.parametrize("what", ["parallel arc", "s-t arc", "far arc", "wrap"])
 @pytest.mark.parametrize("which", sorted(GRIDS))
 def test_almost_lattices_run_the_list_solver(gpu, which, what):
     g = GRIDS[which]()
