@@ -103,6 +103,8 @@ def test_unions_of_one_are_not_prepared_as_lattices(gpu):
     csr = gpu.build_csr(g.n, g.tail, g.head, g.cap)
     other = gpu.build_csr(g.n, np.append(g.tail, g.s), np.append(g.head, g.t), np.append(g.cap, 5).astype(np.int32))
     used = []
+    with gpu.Batch([other], [(g.s, g.t)]):  # the library's code is on the device before memory is looked at
+        pass
     for c in (csr, other):  # the second is no lattice
         torch.cuda.synchronize()
         before = torch.cuda.mem_get_info()[0]
@@ -148,6 +150,11 @@ def test_tiles_take_memory_only_while_options_use_them(gpu):
     g = grid((40000, 8), 6)
     csr = gpu.build_csr(g.n, g.tail, g.head, g.cap)
     lists = dict(max_rounds=2_000_000)  # the default limit, named: a list solve
+    small = grid((40, 30), 7)
+    warm = gpu.build_csr(small.n, small.tail, small.head, small.cap)
+    for o in ({}, lists):  # both solvers' code is on the device before memory is looked at
+        with gpu.Graph.from_csr(warm, small.s, small.t, gpu.default_options(**o)) as G:
+            G.solve()
     torch.cuda.synchronize()
 
     def free():
